@@ -340,6 +340,7 @@ def prepare(case, seed):
         m.integrate(pts[-1], poses[-1])
         row = (3, 3) if kind == "mesh" else (4,)
         st["out"] = torch.zeros((_capacity(case), *row), dtype=torch.float32, device="cuda")
+        st["mine"] = torch.zeros_like(st["out"])
         st["odd"] = torch.randint(-2**62, 2**62, (math.prod(row),), device="cuda",
                                   generator=torch.Generator(device="cuda").manual_seed(1)) * 2 + 1
     return st
@@ -360,11 +361,15 @@ def _serve(st):
     return b.tsdf_server_wait_many(st["server"].value, tickets)
 
 
-def _ordered(rows, odd):
-    """Triangles or points in an order of their own: the library's order is unspecified, and a program that
-    compares, caches or stores them wants the same one each time. Ordered by a hash of their bits."""
-    key = (rows.reshape(rows.shape[0], -1).view(torch.int32) * odd).sum(1)
-    return rows[torch.argsort(key)]
+def _ordered(st, n):
+    """The first n triangles or points in an order of their own, in a buffer kept for them: the library's order is
+    unspecified, and a program that compares, caches or stores them wants the same one each time. Ordered by a
+    hash of their bits."""
+    rows = st["out"].reshape(st["out"].shape[0], -1)[:n]
+    order = torch.argsort((rows.view(torch.int32) * st["odd"]).sum(1))
+    wide = (lambda v: v.view(torch.complex128).reshape(-1)) if rows.shape[1] == 4 else (lambda v: v)   # 16-byte rows move whole
+    torch.index_select(wide(rows), 0, order, out=wide(st["mine"].reshape(st["mine"].shape[0], -1)[:rows.shape[0]]))
+    return st["mine"]
 
 
 def run(st):
@@ -388,10 +393,10 @@ def run(st):
         return dict(counters=[r["stats"]["hits"] for r in _serve(st)], grids=st["grids"])
     if kind == "mesh":
         _, n = b.tsdf_extract_mesh(st["map"].handle, 1, st["out"])
-        return dict(count=n, triangles=_ordered(st["out"], st["odd"]))
+        return dict(count=n, triangles=_ordered(st, n))
     if kind == "surface":
         _, n = b.tsdf_extract_surface(st["map"].handle, 1, st["out"])
-        return dict(count=n, points=_ordered(st["out"], st["odd"]))
+        return dict(count=n, points=_ordered(st, n))
     if kind == "register":
         # the system at the guess (is it worth refining?), then the refinement
         first = b.tsdf_register_system(st["map"].handle, st["pts"], st["pose"])
