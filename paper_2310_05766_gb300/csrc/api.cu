@@ -147,6 +147,7 @@ struct tsdf_map {
     cudaGraphNode_t node_contrib = nullptr;
     cudaKernelNodeParams kp_rays{};
     cudaKernelNodeParams kp_contrib{};
+    bool chain_fused = false;
     MapDev chain_dev{};             // the buffers and options the graph was captured with
     int chain_kpt = 0;
     bool chain_merge = false;
@@ -742,8 +743,14 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         return false;
     }
     const MapDev& d = map->dev;
-    cudaError_t e = launch_rays(a, d, false, true, map->pdl, cs);
-    if (e == cudaSuccess) e = launch_contrib(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
+    const bool fused = scan_fused(a.n);
+    cudaError_t e = cudaSuccess;
+    if (fused) {
+        e = launch_scan(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
+    } else {
+        e = launch_rays(a, d, false, true, map->pdl, cs);
+        if (e == cudaSuccess) e = launch_contrib(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
+    }
     if (e == cudaSuccess) e = launch_compact(d, (uint32_t)map->bricks, map->pdl, cs);
     if (e == cudaSuccess) e = launch_apply(d, map->p.reduce, map->p.w_max, map->p.flags, map->pdl, cs);
     cudaGraph_t g = nullptr;
@@ -753,9 +760,11 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         cudaGetLastError();
         return false;
     }
-    // the two kernel nodes whose arguments change from scan to scan
-    const void* fr = rays_kernel_fn(false, true);
-    const void* fc = contrib_kernel_fn(map->p.reduce, map->merge, map->kpt);
+    // the kernel nodes whose arguments change from scan to scan: the one kernel
+    // of a small scan (kept as the contribution node), or ray set-up and
+    // contribution
+    const void* fr = fused ? nullptr : rays_kernel_fn(false, true);
+    const void* fc = fused ? scan_kernel_fn(map->p.reduce, map->merge) : contrib_kernel_fn(map->p.reduce, map->merge);
     size_t nn = 0;
     std::vector<cudaGraphNode_t> nodes;
     if (cudaGraphGetNodes(g, nullptr, &nn) == cudaSuccess && nn > 0) {
@@ -776,7 +785,7 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         }
     }
     cudaGraphExec_t x = nullptr;
-    if (!map->node_rays || !map->node_contrib || cudaGraphInstantiate(&x, g, 0) != cudaSuccess) {
+    if ((!fused && !map->node_rays) || !map->node_contrib || cudaGraphInstantiate(&x, g, 0) != cudaSuccess) {
         map->node_rays = map->node_contrib = nullptr;
         cudaGraphDestroy(g);
         cudaGetLastError();
@@ -788,6 +797,7 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
     map->chain_kpt = map->kpt;
     map->chain_merge = map->merge;
     map->chain_pdl = map->pdl;
+    map->chain_fused = fused;
     return true;
 }
 
@@ -805,22 +815,28 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
     if (cap != cudaStreamCaptureStatusNone) return TSDF_OK;
     if (map->chain_exec && (!same_dev(map->chain_dev, map->dev) ||
                             map->chain_kpt != map->kpt || map->chain_merge != map->merge ||
-                            map->chain_pdl != map->pdl))
+                            map->chain_pdl != map->pdl || map->chain_fused != scan_fused(a.n)))
         chain_graph_reset(map);
     if (!map->chain_exec && !chain_graph_build(map, a)) {
         map->graph_broken = true;
         return TSDF_OK;
     }
-    void* args[2] = {const_cast<ScanArgs*>(&a), &map->dev};
-    cudaKernelNodeParams kr = map->kp_rays;
-    kr.gridDim = dim3(rays_grid(a.n, false));
-    kr.kernelParams = args;
-    kr.extra = nullptr;
+    ScanShape g = scan_shape(a.n, a.K);
+    void* fused_args[5] = {const_cast<ScanArgs*>(&a), &map->dev, &g.tile, &g.parts, &map->kpt};
+    void* list_args[3] = {const_cast<ScanArgs*>(&a), &map->dev, &map->kpt};   // (the ray set-up takes the first two)
     cudaKernelNodeParams kc = map->kp_contrib;
-    kc.kernelParams = args;
+    kc.kernelParams = map->chain_fused ? fused_args : list_args;
     kc.extra = nullptr;
-    if (cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_rays, &kr) != cudaSuccess ||
-        cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_contrib, &kc) != cudaSuccess) {
+    if (map->chain_fused) kc.gridDim = dim3(g.grid);
+    cudaError_t e = cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_contrib, &kc);
+    if (e == cudaSuccess && !map->chain_fused) {
+        cudaKernelNodeParams kr = map->kp_rays;
+        kr.gridDim = dim3(rays_grid(a.n, false));
+        kr.kernelParams = list_args;
+        kr.extra = nullptr;
+        e = cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_rays, &kr);
+    }
+    if (e != cudaSuccess) {
         cudaGetLastError();
         chain_graph_reset(map);
         map->graph_broken = true;
@@ -833,13 +849,13 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
 
 static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12], cudaStream_t s,
                           int reduction) {
-    int rc = ensure_rays(map, n);
-    if (rc != TSDF_OK) return rc;
+    int rc = TSDF_OK;
     ScanArgs a;
     fill_scan_args(map, points_dev, n, pose, a);
     const bool pdl = map->pdl;
     if (reduction == TSDF_REDUCTION_POOL) {
-        rc = ensure_pool(map);
+        rc = ensure_rays(map, n);
+        if (rc == TSDF_OK) rc = ensure_pool(map);
         if (rc != TSDF_OK) return rc;
         const MapDev& d = map->dev;
         cudaEvent_t e0 = n > 0 ? prof_mark(map, s) : nullptr;
@@ -859,7 +875,8 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
     rc = ensure_acc(map);
     if (rc != TSDF_OK) return rc;
     if (reduction == TSDF_REDUCTION_SORT) {
-        rc = ensure_sort(map, n);
+        rc = ensure_rays(map, n);
+        if (rc == TSDF_OK) rc = ensure_sort(map, n);
         if (rc != TSDF_OK) return rc;
         const MapDev& d = map->dev;
         cudaEvent_t e0 = n > 0 ? prof_mark(map, s) : nullptr;
@@ -883,16 +900,25 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
         prof_push(map, kApply, e6, e7);
         return TSDF_OK;
     }
+    const bool fused = scan_fused(n);
+    if (!fused) {
+        rc = ensure_rays(map, n);
+        if (rc != TSDF_OK) return rc;
+    }
     if (n > 0 && map->use_graph && !map->graph_broken && !map->prof) {
         bool launched = false;
         rc = chain_graph_launch(map, a, s, &launched);
         if (launched || rc != TSDF_OK) return rc;
     }
-    cudaEvent_t e0 = n > 0 ? prof_mark(map, s) : nullptr;
-    TSDF_CU(launch_rays(a, map->dev, false, true, pdl, s));
-    cudaEvent_t e1 = n > 0 ? prof_mark(map, s) : nullptr;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (!fused) {
+        e0 = prof_mark(map, s);
+        TSDF_CU(launch_rays(a, map->dev, false, true, pdl, s));
+        e1 = prof_mark(map, s);
+    }
     cudaEvent_t e2 = n > 0 ? prof_mark(map, s) : nullptr;
-    TSDF_CU(launch_contrib(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s));
+    TSDF_CU(fused ? launch_scan(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s)
+                  : launch_contrib(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s));
     cudaEvent_t e3 = n > 0 ? prof_mark(map, s) : nullptr;
     cudaEvent_t e4 = prof_mark(map, s);
     TSDF_CU(launch_compact(map->dev, (uint32_t)map->bricks, pdl, s));

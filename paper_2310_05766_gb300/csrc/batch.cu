@@ -283,15 +283,15 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
             if (SORT) {
                 const uint32_t sslot = ray < nl ? im.ray_slot[ray] : kNoSlot;
                 if (it.reduce == 0)
-                    contrib_item<0, false, KPT, true>(ia, im, local % ngrp, A, B, hits, last_brick, sslot, &ovf,
+                    contrib_item<0, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
                                                       nullptr, bc);
-                else contrib_item<1, false, KPT, true>(ia, im, local % ngrp, A, B, hits, last_brick, sslot, &ovf,
+                else contrib_item<1, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
                                                        nullptr, bc);
             } else {
                 if (it.reduce == 0)
-                    contrib_item<0, MERGE, KPT>(ia, im, local % ngrp, A, B, hits, last_brick, kNoSlot, nullptr,
+                    contrib_item<0, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
                                                 nullptr, bc);
-                else contrib_item<1, MERGE, KPT>(ia, im, local % ngrp, A, B, hits, last_brick, kNoSlot, nullptr,
+                else contrib_item<1, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
                                                  nullptr, bc);
             }
         }

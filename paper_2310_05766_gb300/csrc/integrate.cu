@@ -27,6 +27,7 @@
 //   shared-memory cache of the bricks the CTA has marked. The items of the
 //   list's front (the costly rays) come first. Integer accumulation makes the
 //   result independent of the order of the atomics.
+// scan: rays and contrib in one kernel, for small scans (scan_fused).
 // compact: turns the brick flags into a list of touched bricks (4 flags per
 //   thread, one list atomic per warp) and clears the flags.
 // apply (K-C): warp tasks over the listed bricks (grid-stride), by default a
@@ -58,17 +59,39 @@
 // Every float operation on the geometry path is an explicit round-to-nearest
 // intrinsic (no contraction into FMA), in the same order as the CPU oracle, so
 // voxel indices and codes agree bit for bit.
+#include <algorithm>
 #include <mutex>
 #include <unordered_map>
 #include <utility>
 
 #include "integrate_device.cuh"
 
-// Minimum resident CTAs per SM requested for the plain contribution kernel:
-// 4 caps it at 64 registers (no spills), 32 resident warps per SM instead of
-// 24 at its natural 79 registers; 34.6 against 35.5 us per outdoor scan.
+// Minimum resident CTAs per SM requested for the scan kernel: 4 caps it at 64
+// registers (no spills), 32 resident warps per SM.
+#ifndef TSDF_SCAN_MIN_CTAS
+#define TSDF_SCAN_MIN_CTAS 4
+#endif
+// The same for the contribution kernel.
 #ifndef TSDF_CONTRIB_MIN_CTAS
 #define TSDF_CONTRIB_MIN_CTAS 4
+#endif
+// Largest scan of the one-kernel path (points). Above it a scan's tiles differ
+// too much in cost for the chip to be filled evenly by whole tiles, and the
+// global ray list, whose 32-ray blocks all march, is the better one. Passes of
+// both paths, one kernel / ray list, in us: room 16x360 17.9 / 26.2 and 64x512
+// 17.2 / 18.1; outdoor 16x512 21.1 / 33.1, 32x512 18.6 / 24.6, 32x1024 34.3 /
+// 38.0, 64x1024 31.3 / 29.4, 128x1024 30.0 / 26.9; corridor 32x512 38.5 / 49.5,
+// 64x1024 41.9 / 44.9, 128x2048 52.1 / 51.4.
+#ifndef TSDF_SCAN_FUSED_MAX
+#define TSDF_SCAN_FUSED_MAX 32768
+#endif
+// Tiles wanted of a scan (six per SM: with three, outdoor 32x512 20.3 instead
+// of 18.6 us, 32x1024 42.1 instead of 34.3), and the largest tile.
+#ifndef TSDF_SCAN_TILES
+#define TSDF_SCAN_TILES 912
+#endif
+#ifndef TSDF_SCAN_MAX_TILE
+#define TSDF_SCAN_MAX_TILE 256
 #endif
 // The same for the sort reduction's emit kernel (no cap).
 #ifndef TSDF_EMIT_MIN_CTAS
@@ -81,15 +104,6 @@
 #endif
 #ifndef TSDF_APPLY_CTAS_PER_SM
 #define TSDF_APPLY_CTAS_PER_SM 0
-#endif
-// 1: the plain path splits its ray list into heavy and light rays (see
-// rays_task); 0: one list in arrival order.
-#ifndef TSDF_RAYS_SPLIT
-#define TSDF_RAYS_SPLIT 1
-#endif
-// Threads per CTA of the contribution kernel.
-#ifndef TSDF_CONTRIB_THREADS
-#define TSDF_CONTRIB_THREADS 256
 #endif
 // Minimum resident CTAs per SM requested for the apply kernel.
 #ifndef TSDF_APPLY_MIN_CTAS
@@ -132,11 +146,12 @@ __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, co
 // brick cache absorbs most marks: giving a CTA's warps unrelated items, or
 // handing out items through counters, made the kernel about 30 % slower, the
 // extra time in brick-flag stores.
-constexpr int kContribThreads = TSDF_CONTRIB_THREADS;
+constexpr int kContribThreads = 256;
 
-template <int MODE, bool MERGE, int KPT>
+template <int MODE, bool MERGE>
 __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contrib_kernel(const ScanArgs a,
-                                                                                        const MapDev m) {
+                                                                                        const MapDev m,
+                                                                                        const int kpt) {
     __shared__ unsigned long long red[kContribThreads / 32];
     __shared__ uint32_t btab[kBrickCache];
     const unsigned lane = threadIdx.x & 31u;
@@ -160,7 +175,7 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     __syncthreads();   // (also orders the brick cache initialisation)
     const unsigned nf = s_counts[0], nb = s_counts[1];
     const unsigned bf = (nf + 31u) / 32u, bb = (nb + 31u) / 32u;
-    const unsigned ngrp = (unsigned)(2 * a.K + KPT) / KPT;   // ceil((2K+1) / KPT)
+    const unsigned ngrp = (unsigned)(2 * a.K + kpt) / (unsigned)kpt;   // ceil((2K+1) / kpt)
     const unsigned nitems = (bf + bb) * ngrp;
     // first ray of block `blk` and the end of its part of the list
     auto block_ray = [&](unsigned blk, unsigned& end) {
@@ -186,13 +201,125 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
         unsigned end;
         const unsigned r0 = block_ray(next / ngrp, end);
         load_rays(m, next < nitems ? end : 0u, r0 + lane, An, Bn);   // prefetch
-        contrib_item<MODE, MERGE, KPT>(a, m, item % ngrp, A, B, hits, last_brick, kNoSlot, nullptr, nullptr, bc);
+        contrib_item<MODE, MERGE>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
+                                                      nullptr, bc);
         A = An;
         B = Bn;
     }
     if (MODE == 1) {
         // MIN_ABS keeps no contribution count per voxel: count them here
         const unsigned long long total = cta_sum<kContribThreads / 32>((unsigned long long)hits, red);
+        if (threadIdx.x == 0 && total) atomicAdd(&m.ctr->part[blockIdx.x % kParts].hits, total);
+    }
+}
+
+constexpr int kScanWarps = 8;
+constexpr int kScanThreads = kScanWarps * 32;
+
+// scan: ray set-up and contributions of one tile of `tile` points (a power of
+// two, 32 .. 256) per CTA; `parts` CTAs share a tile's march steps when the
+// scan has too few tiles for the chip (part p takes every parts-th item, and
+// each of them sets the tile's rays up again).
+//
+// For small scans, which are bound by the chain of kernels and not by work:
+// the rays stay in shared memory, so there is no ray list in memory, no list
+// atomic and one kernel boundary less (the set-up runs before the wait for the
+// previous scan). The tile shrinks with the scan and the work items with the
+// tile, so that a scan of a few thousand points still occupies every SM (a
+// 5760-point scan: 180 CTAs of one 32-ray block, nine steps over eight warps;
+// through the ray list 14.3 us of contributions, here 12.0 with the set-up,
+// and 17.9 instead of 26.2 us for the whole scan).
+template <int MODE, bool MERGE>
+__global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(const ScanArgs a, const MapDev m,
+                                                                               const int tile, const int parts,
+                                                                               const int kpt_max) {
+    __shared__ float4 s_a[kScanThreads], s_b[kScanThreads];
+    __shared__ uint32_t btab[kBrickCache];
+    __shared__ unsigned s_heavy[kScanWarps], s_light[kScanWarps], s_valid[kScanWarps];
+    __shared__ unsigned s_next;
+    __shared__ unsigned long long red[kScanWarps];
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned warp = threadIdx.x >> 5;
+    const unsigned part = parts > 1 ? blockIdx.x % (unsigned)parts : 0u;
+    const int first = (int)(parts > 1 ? blockIdx.x / (unsigned)parts : blockIdx.x) * tile;
+    // ---- the tile's rays, compacted into shared memory
+    const int i = first + (int)threadIdx.x;
+    const bool in = (int)threadIdx.x < tile && i < a.n;
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (in) p = __ldg(a.pts + i);   // the caller's points: no dependency on earlier grids
+    pdl_trigger();
+    brick_cache_init(btab);
+    if (threadIdx.x == 0) s_next = kScanWarps;
+    unsigned nlive, nheavy;
+    {
+        float4 ra, rb;
+        bool valid, live;
+        ray_setup(a, p, in, ra, rb, valid, live);
+        const bool heavy = live && rb.w != 0.f && fm(fm(a.dz, ra.w), a.inv_vs) >= 1.f;
+        const unsigned hmask = __ballot_sync(kFull, heavy);
+        const unsigned lmask = __ballot_sync(kFull, live && !heavy);
+        const unsigned vmask = __ballot_sync(kFull, valid);
+        if (lane == 0) {
+            s_heavy[warp] = __popc(hmask);
+            s_light[warp] = __popc(lmask);
+            s_valid[warp] = __popc(vmask);
+        }
+        __syncthreads();
+        unsigned hb = 0, lb = 0, ht = 0, lt = 0;
+#pragma unroll
+        for (int w = 0; w < kScanWarps; ++w) {
+            const unsigned h = s_heavy[w], l = s_light[w];
+            if (w < (int)warp) {
+                hb += h;
+                lb += l;
+            }
+            ht += h;
+            lt += l;
+        }
+        nheavy = ht;
+        nlive = ht + lt;
+        const unsigned below = (1u << lane) - 1u;
+        if (live) {
+            const unsigned off = heavy ? hb + __popc(hmask & below) : ht + lb + __popc(lmask & below);
+            s_a[off] = ra;
+            s_b[off] = rb;
+        }
+        __syncthreads();
+    }
+    pdl_wait();   // the previous scan's apply resets the counters, flags and accumulators
+    if (part == 0u && threadIdx.x < 32) {
+        const unsigned v = __reduce_add_sync(kFull, lane < kScanWarps ? s_valid[lane] : 0u);
+        if (lane == 0 && v) atomicAdd(&m.ctr->part[blockIdx.x % kParts].valid, (unsigned long long)v);
+    }
+    if (nlive == 0u) return;   // CTA-uniform
+    // ---- march: items (32 rays of the tile, kpt steps), claimed by the warps
+    const unsigned steps = (unsigned)(2 * a.K + 1);
+    const unsigned blocks = (nlive + 31u) / 32u;
+    int kpt = kpt_max;
+    while (kpt > 1 && blocks * ((steps + kpt - 1) / kpt) < 2u * kScanWarps * (unsigned)parts) kpt >>= 1;
+    const unsigned ngrp = (steps + kpt - 1) / kpt;
+    const unsigned nitems = blocks * ngrp;
+    unsigned hits = 0;
+    unsigned last_brick = kNoVoxel;
+    const BrickCache bc{btab, 32u - kBrickCacheLog2};
+    unsigned claim = warp;
+    for (;;) {
+        const unsigned item = claim * (unsigned)parts + part;
+        if (item >= nitems) break;
+        const unsigned ray = (item / ngrp) * 32u + lane;
+        float4 A = make_float4(0.f, 0.f, 0.f, -1.f), B = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ray < nlive) {
+            A = s_a[ray];
+            B = s_b[ray];
+        }
+        contrib_item<MODE, MERGE>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
+                                                      nullptr, bc);
+        if (lane == 0) claim = atomicAdd(&s_next, 1u);
+        claim = __shfl_sync(kFull, claim, 0);
+    }
+    if (MODE == 1) {
+        // MIN_ABS keeps no contribution count per voxel: count them here
+        const unsigned long long total = cta_sum<kScanWarps>((unsigned long long)hits, red);
         if (threadIdx.x == 0 && total) atomicAdd(&m.ctr->part[blockIdx.x % kParts].hits, total);
     }
 }
@@ -222,7 +349,7 @@ __global__ void __launch_bounds__(256, TSDF_EMIT_MIN_CTAS) emit_kernel(const Sca
         float4 A, B;
         load_rays(m, nlive, ray, A, B);
         const uint32_t sslot = ray < nlive ? m.ray_slot[ray] : kNoSlot;
-        contrib_item<MODE, false, KPT, true>(a, m, item % ngrp, A, B, hits, last_brick, sslot, &ovf, nullptr,
+        contrib_item<MODE, false, true>(a, m, item % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf, nullptr,
                                              BrickCache{btab, 32u - kBrickCacheLog2});
     }
     if (ovf) m.ctr->overflow = 1u;
@@ -253,7 +380,7 @@ __global__ void __launch_bounds__(256) pool_contrib_kernel(const ScanArgs a, con
     for (unsigned item = gwarp; item < nitems; item += nwarps) {   // warp-uniform
         float4 A, B;
         load_rays(m, nlive, (item / ngrp) * 32u + lane, A, B);
-        contrib_item<MODE, false, KPT, false, true>(a, m, item % ngrp, A, B, hits, last_brick, kNoSlot, nullptr,
+        contrib_item<MODE, false, false, true>(a, m, item % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
                                                     &last_slot);
     }
     if (MODE == 1) {
@@ -528,22 +655,6 @@ dim3 resident_grid(void (*kernel)(KArgs...), int threads, int per_sm = 0) {
     return dim3((unsigned)resident_ctas(reinterpret_cast<const void*>(kernel), threads));
 }
 
-template <int MODE, bool MERGE, int KPT>
-cudaError_t launch_contrib_kk(const ScanArgs& a, const MapDev& m, bool pdl, cudaStream_t s) {
-    auto* k = contrib_kernel<MODE, MERGE, KPT>;
-    return launch(k, resident_grid(k, kContribThreads, TSDF_CONTRIB_CTAS_PER_SM), dim3(kContribThreads), s, pdl, a,
-                  m);
-}
-
-template <int MODE, bool MERGE>
-cudaError_t launch_contrib_k(const ScanArgs& a, const MapDev& m, int kpt, bool pdl, cudaStream_t s) {
-    switch (kpt) {
-        case 2: return launch_contrib_kk<MODE, MERGE, 2>(a, m, pdl, s);
-        case 4: return launch_contrib_kk<MODE, MERGE, 4>(a, m, pdl, s);
-        default: return launch_contrib_kk<MODE, MERGE, 1>(a, m, pdl, s);
-    }
-}
-
 template <int MODE, int KPT>
 cudaError_t launch_emit_k(const ScanArgs& a, const MapDev& m, bool pdl, cudaStream_t s) {
     auto* k = emit_kernel<MODE, KPT>;
@@ -552,28 +663,54 @@ cudaError_t launch_emit_k(const ScanArgs& a, const MapDev& m, bool pdl, cudaStre
 
 }  // namespace
 
-const void* rays_kernel_fn(bool sort, bool split) {
-    if (sort) return reinterpret_cast<const void*>(rays_kernel<true, false>);
-    return split && TSDF_RAYS_SPLIT ? reinterpret_cast<const void*>(rays_kernel<false, true>)
-                                    : reinterpret_cast<const void*>(rays_kernel<false, false>);
+// Tile and parts of a scan of n points with K march steps each side of the hit.
+// The largest tile that gives every SM work (several CTAs for each, so that
+// uneven tiles even out); with the smallest tile, several CTAs per tile while
+// each still has an item for every warp.
+bool scan_fused(int64_t n) { return n <= TSDF_SCAN_FUSED_MAX; }
+
+ScanShape scan_shape(int64_t n, int K) {
+    const int64_t want = TSDF_SCAN_TILES;
+    ScanShape g{TSDF_SCAN_MAX_TILE, 1, 0};
+    while (g.tile > 32 && (n + g.tile - 1) / g.tile < want) g.tile >>= 1;
+    const int64_t tiles = (n + g.tile - 1) / g.tile;
+    if (tiles > 0 && tiles < want) {
+        const int64_t items = (int64_t)(g.tile / 32) * (2 * (int64_t)K + 1);
+        g.parts = (int)std::max<int64_t>(1, std::min<int64_t>((want + tiles - 1) / tiles, items / kScanWarps));
+    }
+    g.grid = (unsigned)(tiles * g.parts);
+    return g;
 }
 
-const void* contrib_kernel_fn(int32_t reduce, bool merge, int kpt) {
-    const int k = kpt == 2 || kpt == 4 ? kpt : 1;
-    if (reduce == 0) {
-        if (merge) return k == 4 ? reinterpret_cast<const void*>(contrib_kernel<0, true, 4>)
-                        : k == 2 ? reinterpret_cast<const void*>(contrib_kernel<0, true, 2>)
-                                 : reinterpret_cast<const void*>(contrib_kernel<0, true, 1>);
-        return k == 4 ? reinterpret_cast<const void*>(contrib_kernel<0, false, 4>)
-             : k == 2 ? reinterpret_cast<const void*>(contrib_kernel<0, false, 2>)
-                      : reinterpret_cast<const void*>(contrib_kernel<0, false, 1>);
-    }
-    if (merge) return k == 4 ? reinterpret_cast<const void*>(contrib_kernel<1, true, 4>)
-                    : k == 2 ? reinterpret_cast<const void*>(contrib_kernel<1, true, 2>)
-                             : reinterpret_cast<const void*>(contrib_kernel<1, true, 1>);
-    return k == 4 ? reinterpret_cast<const void*>(contrib_kernel<1, false, 4>)
-         : k == 2 ? reinterpret_cast<const void*>(contrib_kernel<1, false, 2>)
-                  : reinterpret_cast<const void*>(contrib_kernel<1, false, 1>);
+const void* scan_kernel_fn(int32_t reduce, bool merge) {
+    if (reduce == 0)
+        return merge ? reinterpret_cast<const void*>(scan_kernel<0, true>)
+                     : reinterpret_cast<const void*>(scan_kernel<0, false>);
+    return merge ? reinterpret_cast<const void*>(scan_kernel<1, true>)
+                 : reinterpret_cast<const void*>(scan_kernel<1, false>);
+}
+
+cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
+                        cudaStream_t s) {
+    if (a.n <= 0) return cudaSuccess;
+    const ScanShape g = scan_shape(a.n, a.K);
+    auto* k = reduce == 0 ? (merge ? scan_kernel<0, true> : scan_kernel<0, false>)
+                          : (merge ? scan_kernel<1, true> : scan_kernel<1, false>);
+    return launch(k, dim3(g.grid), dim3(kScanThreads), s, pdl, a, m, g.tile, g.parts, kpt);
+}
+
+const void* rays_kernel_fn(bool sort, bool split) {
+    if (sort) return reinterpret_cast<const void*>(rays_kernel<true, false>);
+    return split ? reinterpret_cast<const void*>(rays_kernel<false, true>)
+                 : reinterpret_cast<const void*>(rays_kernel<false, false>);
+}
+
+const void* contrib_kernel_fn(int32_t reduce, bool merge) {
+    if (reduce == 0)
+        return merge ? reinterpret_cast<const void*>(contrib_kernel<0, true>)
+                     : reinterpret_cast<const void*>(contrib_kernel<0, false>);
+    return merge ? reinterpret_cast<const void*>(contrib_kernel<1, true>)
+                 : reinterpret_cast<const void*>(contrib_kernel<1, false>);
 }
 
 unsigned rays_grid(int64_t n, bool sort) {
@@ -585,8 +722,17 @@ cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool spli
     if (a.n <= 0) return cudaSuccess;
     const dim3 grid(rays_grid(a.n, sort)), block(kRaysThreads);
     if (sort) return launch(rays_kernel<true, false>, grid, block, s, pdl, a, m);
-    return split && TSDF_RAYS_SPLIT ? launch(rays_kernel<false, true>, grid, block, s, pdl, a, m)
-                                    : launch(rays_kernel<false, false>, grid, block, s, pdl, a, m);
+    return split ? launch(rays_kernel<false, true>, grid, block, s, pdl, a, m)
+                 : launch(rays_kernel<false, false>, grid, block, s, pdl, a, m);
+}
+
+cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
+                           cudaStream_t s) {
+    if (a.n <= 0) return cudaSuccess;
+    auto* k = reduce == 0 ? (merge ? contrib_kernel<0, true> : contrib_kernel<0, false>)
+                          : (merge ? contrib_kernel<1, true> : contrib_kernel<1, false>);
+    return launch(k, resident_grid(k, kContribThreads, TSDF_CONTRIB_CTAS_PER_SM), dim3(kContribThreads), s, pdl, a, m,
+                  kpt);
 }
 
 cudaError_t launch_emit(const ScanArgs& a, const MapDev& m, int32_t reduce, int kpt, bool pdl, cudaStream_t s) {
@@ -646,14 +792,6 @@ cudaError_t launch_sort_apply(const MapDev& m, int32_t reduce, int32_t w_max, in
     auto* k = reduce == 0 ? sort_apply_kernel<0> : sort_apply_kernel<1>;
     return launch(k, resident_grid(k, kApplyWarps * 32, TSDF_APPLY_CTAS_PER_SM), dim3(kApplyWarps * 32), s, pdl, m,
                   w_max, flags);
-}
-
-cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
-                           cudaStream_t s) {
-    if (a.n <= 0) return cudaSuccess;
-    if (reduce == 0)
-        return merge ? launch_contrib_k<0, true>(a, m, kpt, pdl, s) : launch_contrib_k<0, false>(a, m, kpt, pdl, s);
-    return merge ? launch_contrib_k<1, true>(a, m, kpt, pdl, s) : launch_contrib_k<1, false>(a, m, kpt, pdl, s);
 }
 
 cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStream_t s) {

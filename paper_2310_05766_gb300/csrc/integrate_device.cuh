@@ -32,9 +32,6 @@ __device__ __forceinline__ void brick_cache_init(uint32_t* btab) {
     for (int i = threadIdx.x; i < kBrickCache; i += blockDim.x) btab[i] = kNoVoxel;
 }
 
-#ifndef TSDF_MARK_SHFL
-#define TSDF_MARK_SHFL 0
-#endif
 // 1: the plain atomic contribution march runs lean_march (fewer instructions
 // per sample, same results); 0: the general march
 #ifndef TSDF_LEAN_MARCH
@@ -104,7 +101,6 @@ struct RaysSmemT {
     unsigned bbase;                 // split list: the CTA's first light-ray entry, counted from the end
     unsigned long long sbase;       // the CTA's first pair slot (sort reduction)
 };
-using RaysSmem = RaysSmemT<8>;
 
 // One point of a scan (sensor frame; `in`: the point exists): world transform,
 // range test, unit direction, fill direction (Eq. 3 / Eq. 4) and the
@@ -350,7 +346,7 @@ __device__ __forceinline__ void load_rays(const MapDev& m, unsigned end, unsigne
     }
 }
 
-// One warp: the steps of k-group `grp` (KPT steps) of its 32 rays.
+// One warp: the steps of k-group `grp` (kpt steps) of its 32 rays.
 // SORT (sort reduction, MERGE off): each sample of a lane's ray is written to
 // the ray's pair slot sslot + (its index in the ray's march) instead of being
 // reduced: (voxel word, code) inside the window, kNoVoxel outside. Samples
@@ -405,6 +401,28 @@ __device__ __forceinline__ uint32_t pool_slot(const MapDev& m, unsigned brick) {
         }
     }
     return __shfl_sync(peers, s, leader);
+}
+
+// A contribution falls into `brick`: store its flag byte (idempotent, nothing
+// to wait for; same-address byte stores of a warp merge into one transaction).
+// With a brick cache only on a cache miss: many lanes and warps touch the same
+// few bricks, and same-address stores from every SM are what makes the marking
+// costly. (Any thread that puts a brick into the cache also stores its flag, so
+// a hit never hides an unmarked brick.) Building the brick list here instead
+// (the CTA's first visitor of a brick queues it with shared-memory atomics, and
+// the CTA lists its queue when it has marched) was measured slower: it saves
+// the compaction kernel's 3 us and costs the outdoor scan's contributions 2.5
+// (an exact open-addressing set of the CTA's bricks: 4 us).
+__device__ __forceinline__ void mark_brick(const MapDev& m, unsigned brick, const BrickCache& bc) {
+    if (bc.tab) {
+        const unsigned h = (brick * 2654435761u) >> bc.shift;
+        if (bc.tab[h] != brick + bc.tag) {
+            bc.tab[h] = brick + bc.tag;
+            m.brick_flag[brick] = 1;
+        }
+    } else {
+        m.brick_flag[brick] = 1;
+    }
 }
 
 // ---- lean march of the plain atomic reduction (no sort, pool or merge).
@@ -491,33 +509,24 @@ __device__ __forceinline__ void lean_sample(const ScanArgs& a, const MapDev& m, 
             atomicMax(m.acc + word, 65536ull - key);
             ++hits;
         }
-        // mark the brick unless this lane marked it last; with a brick cache
-        // the global flag store only on a cache miss (see contrib_item)
+        // mark the brick unless this lane marked it last
         const unsigned brick = word >> 9;
         if (brick != last_brick) {
             last_brick = brick;
-            if (bc.tab) {
-                const unsigned h = (brick * 2654435761u) >> bc.shift;
-                if (bc.tab[h] != brick + bc.tag) {
-                    bc.tab[h] = brick + bc.tag;
-                    m.brick_flag[brick] = 1;
-                }
-            } else {
-                m.brick_flag[brick] = 1;
-            }
+            mark_brick(m, brick, bc);
         }
     }
 }
 
-// The steps k0 .. k0 + KPT - 1 (at most K) of the warp's 32 rays.
-template <int MODE, int KPT, bool SV>
-__device__ __forceinline__ void lean_march(const ScanArgs& a, const MapDev& m, int k0, const float4& A,
+// The steps k0 .. k0 + kpt - 1 (at most K) of the warp's 32 rays.
+template <int MODE, bool SV>
+__device__ __forceinline__ void lean_march(const ScanArgs& a, const MapDev& m, int k0, int kpt, const float4& A,
                                            const float4& B, unsigned& hits, unsigned& last_brick,
                                            const BrickCache& bc) {
     const float r = A.w;                // dead lanes carry r = -1
     const bool rfill = B.w != 0.f;
 #pragma unroll 1
-    for (int kk = 0; kk < KPT; ++kk) {
+    for (int kk = 0; kk < kpt; ++kk) {
         const int k = k0 + kk;
         if (k > a.K) break;   // uniform
         float l;
@@ -540,8 +549,8 @@ __device__ __forceinline__ void lean_march(const ScanArgs& a, const MapDev& m, i
     }
 }
 
-template <int MODE, bool MERGE, int KPT, bool SORT = false, bool POOL = false>
-__device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m, unsigned grp, const float4 A,
+template <int MODE, bool MERGE, bool SORT = false, bool POOL = false>
+__device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m, unsigned grp, int kpt, const float4 A,
                                              const float4 B, unsigned& hits, unsigned& last_brick,
                                              uint32_t sslot = kNoSlot, bool* ovf = nullptr,
                                              uint32_t* last_slot = nullptr, BrickCache bc = BrickCache{}) {
@@ -549,9 +558,9 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
     static_assert(!(POOL && (SORT || MERGE)), "the pool reduction is a variant of the plain atomic one");
 #if TSDF_LEAN_MARCH
     if constexpr (!SORT && !POOL && !MERGE) {
-        const int k0l = (int)grp * KPT - a.K;
-        if (a.flags & kFlagStepValue) lean_march<MODE, KPT, true>(a, m, k0l, A, B, hits, last_brick, bc);
-        else lean_march<MODE, KPT, false>(a, m, k0l, A, B, hits, last_brick, bc);
+        const int k0l = (int)grp * kpt - a.K;
+        if (a.flags & kFlagStepValue) lean_march<MODE, true>(a, m, k0l, kpt, A, B, hits, last_brick, bc);
+        else lean_march<MODE, false>(a, m, k0l, kpt, A, B, hits, last_brick, bc);
         return;
     }
 #endif
@@ -559,7 +568,7 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
     const float tx = a.t[0], ty = a.t[1], tz = a.t[2];
     const float r = A.w;                // dead lanes carry r = -1
     const bool rfill = B.w != 0.f;
-    const int k0 = (int)grp * KPT - a.K;
+    const int k0 = (int)grp * kpt - a.K;
     uint32_t sidx = 0;                  // SORT: index of the step's first sample in the ray's march
     if (SORT && sslot != kNoSlot) {
         for (int k = -a.K; k < k0; ++k) {
@@ -569,7 +578,7 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
         }
     }
 #pragma unroll 1
-    for (int kk = 0; kk < KPT; ++kk) {
+    for (int kk = 0; kk < kpt; ++kk) {
         const int k = k0 + kk;
         if (k > a.K) break;   // uniform
         float l;
@@ -654,30 +663,10 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
                 }
             }
             if (MODE == 1 && !SORT) hits += act ? 1u : 0u;
-            // mark the brick unless this lane marked it last (same-address
-            // byte stores of a warp merge into one transaction); optionally
-            // also skip when the lane below marks the same brick now. With a
-            // brick cache the global store is issued only on a cache miss:
-            // many lanes and warps touch the same few bricks, and same-address
-            // stores from every SM are what makes the marking costly. (Any
-            // thread that puts a brick into the cache also stores its flag,
-            // so a hit never hides an unmarked brick.)
-#if TSDF_MARK_SHFL
-            const unsigned below = __shfl_up_sync(kFull, leader ? brick : kNoVoxel, 1);
-            if (leader && brick != last_brick && (lane == 0 || below != brick)) {
-#else
+            // mark the brick unless this lane marked it last
             if (leader && brick != last_brick) {
-#endif
                 last_brick = brick;
-                if (bc.tab) {
-                    const unsigned h = (brick * 2654435761u) >> bc.shift;
-                    if (bc.tab[h] != brick + bc.tag) {
-                        bc.tab[h] = brick + bc.tag;
-                        m.brick_flag[brick] = 1;
-                    }
-                } else {
-                    m.brick_flag[brick] = 1;
-                }
+                mark_brick(m, brick, bc);
             }
         }
         if (SORT && lv) sidx += 2u * (uint32_t)J + 1u;

@@ -118,8 +118,7 @@ extern "C" int tsdf_integrate_static(uint32_t* grid_dev, const tsdf_params* para
     rc = scratch_for_current_device(&base, &dev);
     if (rc != TSDF_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t voxels = (size_t)params->dims[0] * params->dims[1] * params->dims[2];
-    const size_t bricks = voxels / kBrickVoxels;
+    const size_t bricks = (size_t)params->dims[0] * params->dims[1] * params->dims[2] / kBrickVoxels;
 
     MapDev md{};
     md.grid = grid_dev;
@@ -181,10 +180,14 @@ extern "C" int tsdf_integrate_static(uint32_t* grid_dev, const tsdf_params* para
     a.flags = params->flags;
     fill_lean_args(a);
 
-    if (e == cudaSuccess) e = launch_rays(a, md, false, true, true, s);
     bool launched_contrib = false;
     if (e == cudaSuccess) {
-        e = launch_contrib(a, md, params->reduce, false, 4, true, s);
+        if (scan_fused(n)) {
+            e = launch_scan(a, md, params->reduce, false, 4, true, s);
+        } else {
+            e = launch_rays(a, md, false, true, true, s);
+            if (e == cudaSuccess) e = launch_contrib(a, md, params->reduce, false, 4, true, s);
+        }
         launched_contrib = true;
     }
     if (e == cudaSuccess) e = launch_compact(md, (uint32_t)bricks, true, s);

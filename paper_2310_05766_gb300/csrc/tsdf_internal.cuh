@@ -180,14 +180,27 @@ int map_reserve_sort(::tsdf_map* map, int64_t n);
 // Launchers (return the cudaError_t of the launch).
 // sort: reserve pair slots per ray (sort reduction); split: heavy rays (fill
 // of at least one voxel each side) from the list's front, the others from
-// its end (the plain contribution kernel takes heavy work first).
+// its end (the contribution kernel takes heavy work first).
 cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool split, bool pdl, cudaStream_t s);
+// Plain atomic path up to the list of touched bricks: one kernel over tiles
+// of points for small scans, else ray set-up and the contribution kernel
+// (scan_fused tells which; the ray list is needed only by the latter).
+bool scan_fused(int64_t n);
+struct ScanShape {
+    int tile;                       // points per CTA
+    int parts;                      // CTAs that share a tile's march steps
+    unsigned grid;                  // CTAs
+};
+ScanShape scan_shape(int64_t n, int K);
 // CTAs of the ray set-up kernel for a scan of n points.
 unsigned rays_grid(int64_t n, bool sort);
-// The kernel functions that launch_rays / launch_contrib launch for these
-// arguments (to find their nodes in a captured graph).
+// The kernel functions that these launchers launch for these arguments (to
+// find their nodes in a captured graph).
+const void* scan_kernel_fn(int32_t reduce, bool merge);
 const void* rays_kernel_fn(bool sort, bool split);
-const void* contrib_kernel_fn(int32_t reduce, bool merge, int kpt);
+const void* contrib_kernel_fn(int32_t reduce, bool merge);
+cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
+                        cudaStream_t s);
 cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
                            cudaStream_t s);
 cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStream_t s);
