@@ -553,8 +553,8 @@ int tsdf_map_create(const tsdf_params* params, tsdf_map** out) {
     if (e == cudaSuccess) e = cudaMemset(m->dev.ctr, 0, sizeof(MapCounters));
     // published counters mirrored into mapped pinned memory (falls back to a
     // device-to-host copy in tsdf_stats when the mapping is unavailable)
-    if (e == cudaSuccess && cudaHostAlloc(&m->host_last, 4 * sizeof(long long), cudaHostAllocMapped) == cudaSuccess) {
-        std::memset(m->host_last, 0, 4 * sizeof(long long));
+    if (e == cudaSuccess && cudaHostAlloc(&m->host_last, kPubWords * sizeof(long long), cudaHostAllocMapped) == cudaSuccess) {
+        std::memset(m->host_last, 0, kPubWords * sizeof(long long));
         void* dp = nullptr;
         if (cudaHostGetDevicePointer(&dp, m->host_last, 0) == cudaSuccess) {
             m->dev.host_last = static_cast<long long*>(dp);
@@ -716,7 +716,7 @@ static void fill_scan_args(const tsdf_map* map, const float* points_dev, int64_t
     fill_lean_args(a);
 }
 
-static_assert(sizeof(MapDev) == 160, "same_dev compares every field of MapDev");
+static_assert(sizeof(MapDev) == 168, "same_dev compares every field of MapDev but the parity");
 static bool same_dev(const MapDev& x, const MapDev& y) {
     return x.grid == y.grid && x.acc == y.acc && x.brick_flag == y.brick_flag && x.brick_list == y.brick_list &&
            x.ray_a == y.ray_a && x.ray_b == y.ray_b && x.ray_cap == y.ray_cap && x.ctr == y.ctr &&
@@ -742,7 +742,8 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         cudaGetLastError();
         return false;
     }
-    const MapDev& d = map->dev;
+    MapDev d = map->dev;
+    d.parity = 0;   // graph launches do not overlap: the graph's nodes keep one set of ray counts
     const bool fused = scan_fused(a.n);
     cudaError_t e = cudaSuccess;
     if (fused) {
@@ -751,8 +752,7 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         e = launch_rays(a, d, false, true, map->pdl, cs);
         if (e == cudaSuccess) e = launch_contrib(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
     }
-    if (e == cudaSuccess) e = launch_compact(d, (uint32_t)map->bricks, map->pdl, cs);
-    if (e == cudaSuccess) e = launch_apply(d, map->p.reduce, map->p.w_max, map->p.flags, map->pdl, cs);
+    if (e == cudaSuccess) e = launch_apply(d, (uint32_t)map->bricks, map->p.reduce, map->p.w_max, map->p.flags, map->pdl, cs);
     cudaGraph_t g = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(cs, &g);
     if (e != cudaSuccess || ee != cudaSuccess || !g) {
@@ -822,8 +822,10 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
         return TSDF_OK;
     }
     ScanShape g = scan_shape(a.n, a.K);
-    void* fused_args[5] = {const_cast<ScanArgs*>(&a), &map->dev, &g.tile, &g.parts, &map->kpt};
-    void* list_args[3] = {const_cast<ScanArgs*>(&a), &map->dev, &map->kpt};   // (the ray set-up takes the first two)
+    MapDev d = map->dev;
+    d.parity = 0;
+    void* fused_args[5] = {const_cast<ScanArgs*>(&a), &d, &g.tile, &g.parts, &map->kpt};
+    void* list_args[3] = {const_cast<ScanArgs*>(&a), &d, &map->kpt};   // (the ray set-up takes the first two)
     cudaKernelNodeParams kc = map->kp_contrib;
     kc.kernelParams = map->chain_fused ? fused_args : list_args;
     kc.extra = nullptr;
@@ -843,6 +845,7 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
         return TSDF_OK;
     }
     *launched = true;
+    map->dev.parity = 0;   // (the next plain scan takes the other set)
     TSDF_CU(cudaGraphLaunch(map->chain_exec, s));
     return TSDF_OK;
 }
@@ -910,6 +913,7 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
         rc = chain_graph_launch(map, a, s, &launched);
         if (launched || rc != TSDF_OK) return rc;
     }
+    map->dev.parity ^= 1u;   // this scan's ray counts (see LiveCounts)
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!fused) {
         e0 = prof_mark(map, s);
@@ -921,8 +925,7 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
                   : launch_contrib(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s));
     cudaEvent_t e3 = n > 0 ? prof_mark(map, s) : nullptr;
     cudaEvent_t e4 = prof_mark(map, s);
-    TSDF_CU(launch_compact(map->dev, (uint32_t)map->bricks, pdl, s));
-    TSDF_CU(launch_apply(map->dev, map->p.reduce, map->p.w_max, map->p.flags, pdl, s));   // + counters
+    TSDF_CU(launch_apply(map->dev, (uint32_t)map->bricks, map->p.reduce, map->p.w_max, map->p.flags, pdl, s));
     cudaEvent_t e5 = prof_mark(map, s);
     prof_push(map, kRays, e0, e1);
     prof_push(map, kContrib, e2, e3);
@@ -1194,22 +1197,20 @@ int tsdf_stats(tsdf_map* map, tsdf_scan_stats* out, void* stream) {
     if (!map || !out) return TSDF_ERR_INVALID;
     DeviceScope ds(map->device);
     cudaStream_t s = (cudaStream_t)stream;
-    long long last[3] = {0, 0, 0};   // last_valid, last_hits, last_touched are contiguous
-    static_assert(offsetof(MapCounters, last_touched) == offsetof(MapCounters, last_valid) + 16, "layout");
+    long long last[3] = {0, 0, 0};
     long long status = 0;
-    static_assert(offsetof(MapCounters, last_status) == offsetof(MapCounters, last_valid) + 24, "layout");
     static_assert(kStatusCapacity == TSDF_ERR_CAPACITY, "status code");
     if (map->host_last) {
-        // the last apply CTA of each scan also wrote them to mapped host memory
+        // every scan also writes them to mapped host memory
         TSDF_CU(cudaStreamSynchronize(s));
-        std::memcpy(last, (const void*)map->host_last, sizeof(last));
+        sum_counters(map->host_last, last);
         status = ((volatile long long*)map->host_last)[3];
     } else {
-        long long buf[4] = {0, 0, 0, 0};
-        TSDF_CU(cudaMemcpyAsync(buf, &map->dev.ctr->last_valid, sizeof(buf), cudaMemcpyDeviceToHost, s));
+        long long pub[kPubWords] = {};
+        TSDF_CU(cudaMemcpyAsync(pub, map->dev.ctr->pub, sizeof(pub), cudaMemcpyDeviceToHost, s));
         TSDF_CU(cudaStreamSynchronize(s));
-        std::memcpy(last, buf, sizeof(last));
-        status = buf[3];
+        sum_counters(pub, last);
+        status = pub[3];
     }
     out->valid_rays = last[0];
     out->hits = last[1];
@@ -1732,7 +1733,7 @@ int prepare_batch_item(::tsdf_map* map, const float* points_dev, int64_t n, cons
 
 int map_device(const ::tsdf_map* map) { return map->device; }
 
-const long long* map_last_counters(const ::tsdf_map* map) { return &map->dev.ctr->last_valid; }
+const long long* map_last_counters(const ::tsdf_map* map) { return map->dev.ctr->pub; }
 
 const volatile long long* map_host_counters(const ::tsdf_map* map) { return map->host_last; }
 

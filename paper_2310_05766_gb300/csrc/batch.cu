@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
             p1_map = i;
         }
         if constexpr (SORT)
-            rays_task<false, SORT, false, kBatchWarps>(s_args[0], s_dev[0], (int)((t - hdr->ray_prefix[i]) * THREADS),
+            rays_task_sort<false, kBatchWarps>(s_args[0], s_dev[0], (int)((t - hdr->ray_prefix[i]) * THREADS),
                                                        t, &rsm);
         else
             rays_task_ppt<false, false, kBatchWarps, RPPT>(s_args[0], s_dev[0],

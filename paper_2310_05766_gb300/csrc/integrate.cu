@@ -28,19 +28,20 @@
 //   list's front (the costly rays) come first. Integer accumulation makes the
 //   result independent of the order of the atomics.
 // scan: rays and contrib in one kernel, for small scans (scan_fused).
-// compact: turns the brick flags into a list of touched bricks (4 flags per
-//   thread, one list atomic per warp) and clears the flags.
-// apply (K-C): warp tasks over the listed bricks (grid-stride), by default a
-//   quarter brick per task: each lane loads its voxel pairs' accumulators and
-//   grid words into registers with coalesced loads, applies Eq. 1 in exact
-//   integers with one rounding (half away from zero) and Eq. 2 with the weight
-//   cap to every touched voxel (non-zero accumulator), writes changed pairs
-//   back and resets their accumulators. (TSDF_APPLY_REG 0 selects the older
-//   form: a warp per brick staged in shared memory, touched voxels compacted
-//   with a warp scan.) Touched voxels are counted, and in WSUM mode the
-//   contributions too (the sum of the decoded weights).
-// finish: the last apply CTA to retire sums the per-scan counters into the
-//   published ones and clears the per-scan state (one warp).
+// compact (large windows, sort reduction): turns the brick flags into a list of
+//   touched bricks (4 flags per thread, one list atomic per warp) and clears
+//   the flags.
+// apply (K-C): one CTA per SM; each reads the brick flags itself (windows of
+//   up to 2^16 bricks; the compaction kernel lists the bricks of larger ones),
+//   takes its share of the touched bricks and works on quarter-brick warp
+//   tasks staged through shared memory: Eq. 1 in exact integers with one
+//   rounding (half away from zero) and Eq. 2 with the weight cap for every
+//   touched voxel (non-zero accumulator), changed pairs written back and their
+//   accumulators reset. Each CTA publishes its share of the scan's counters:
+//   touched voxels and, in WSUM mode, the contributions too (the sum of the
+//   decoded weights).
+// finish (the other reductions): the last apply CTA to retire sums the
+//   per-scan counters into the published ones and clears the per-scan state.
 //
 // Sort reduction (an alternative to the accumulator atomics, same results):
 // rays also reserve each live ray's pair slots (one per march sample); emit is
@@ -61,6 +62,7 @@
 // voxel indices and codes agree bit for bit.
 #include <algorithm>
 #include <mutex>
+#include <set>
 #include <unordered_map>
 #include <utility>
 
@@ -97,22 +99,10 @@
 #ifndef TSDF_EMIT_MIN_CTAS
 #define TSDF_EMIT_MIN_CTAS 1
 #endif
-// CTAs per SM launched by the contribution and apply kernels, which walk
-// their work with a grid stride; 0 = as many as are resident at once.
+// CTAs per SM launched by the contribution kernels, which walk their work with
+// a grid stride; 0 = as many as are resident at once.
 #ifndef TSDF_CONTRIB_CTAS_PER_SM
 #define TSDF_CONTRIB_CTAS_PER_SM 8
-#endif
-#ifndef TSDF_APPLY_CTAS_PER_SM
-#define TSDF_APPLY_CTAS_PER_SM 0
-#endif
-// Minimum resident CTAs per SM requested for the apply kernel.
-#ifndef TSDF_APPLY_MIN_CTAS
-#define TSDF_APPLY_MIN_CTAS 1
-#endif
-// 1: the apply kernel keeps each lane's voxels in registers (apply_brick_reg);
-// 0: it stages the brick in shared memory and compacts the touched voxels.
-#ifndef TSDF_APPLY_REG
-#define TSDF_APPLY_REG 1
 #endif
 
 namespace tsdf {
@@ -130,7 +120,7 @@ template <bool SORT, bool SPLIT>
 __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, const MapDev m) {
     __shared__ RaysSmemT<kRaysThreads / 32> sm;
     if constexpr (SORT)
-        rays_task<true, SORT, SPLIT, kRaysThreads / 32>(a, m, (int)(blockIdx.x * blockDim.x), blockIdx.x, &sm);
+        rays_task_sort<true, kRaysThreads / 32>(a, m, (int)(blockIdx.x * blockDim.x), blockIdx.x, &sm);
     else
         rays_task_ppt<true, SPLIT, kRaysThreads / 32, kRaysPPT>(a, m, (int)(blockIdx.x * blockDim.x) * kRaysPPT,
                                                                 blockIdx.x, &sm);
@@ -169,8 +159,8 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     // costly items are taken by the first wave of CTAs and the CTAs that start
     // late get light ones.
     if (threadIdx.x == 0) {
-        s_counts[0] = __ldcg(&m.ctr->live_count);
-        s_counts[1] = __ldcg(&m.ctr->live_back);
+        s_counts[0] = __ldcg(&m.ctr->live[m.parity].front);
+        s_counts[1] = __ldcg(&m.ctr->live[m.parity].back);
     }
     __syncthreads();   // (also orders the brick cache initialisation)
     const unsigned nf = s_counts[0], nb = s_counts[1];
@@ -289,7 +279,7 @@ __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(
     pdl_wait();   // the previous scan's apply resets the counters, flags and accumulators
     if (part == 0u && threadIdx.x < 32) {
         const unsigned v = __reduce_add_sync(kFull, lane < kScanWarps ? s_valid[lane] : 0u);
-        if (lane == 0 && v) atomicAdd(&m.ctr->part[blockIdx.x % kParts].valid, (unsigned long long)v);
+        if (lane == 0 && v) atomicAdd(&m.ctr->live[m.parity].valid, v);
     }
     if (nlive == 0u) return;   // CTA-uniform
     // ---- march: items (32 rays of the tile, kpt steps), claimed by the warps
@@ -423,76 +413,254 @@ __global__ void __launch_bounds__(256) compact_kernel(const MapDev m, const uint
     compact_words(m, blockIdx.x * blockDim.x + threadIdx.x, nwords);
 }
 
-constexpr int kApplyWarps = 4;   // CTA size of the staged (sort and pool) apply kernels
-// CTA size of the register apply kernel.
-#ifndef TSDF_APPLY_WARPS
-#define TSDF_APPLY_WARPS 4
-#endif
-#if TSDF_APPLY_REG
-constexpr int kRegApplyWarps = TSDF_APPLY_WARPS;
-#else
-constexpr int kRegApplyWarps = kApplyWarps;
-#endif
-// Voxel pairs per lane in one apply task: 8 = a warp per brick, 4 = a warp
-// per half brick, 2 = per quarter brick (more, shorter tasks in flight: the
-// apply is latency-bound).
-#ifndef TSDF_APPLY_PAIRS
-#define TSDF_APPLY_PAIRS 2
-#endif
-constexpr int kApplyPairs = TSDF_APPLY_PAIRS;
+constexpr int kApplyWarps = 4;   // CTA size of the sort and pool apply kernels
 
-// The last CTA to finish also publishes the scan's counters (finish_if_last).
-template <int MODE>
-__global__ void __launch_bounds__(kRegApplyWarps * 32, TSDF_APPLY_MIN_CTAS) apply_kernel(const MapDev m,
-                                                                                         const int32_t w_max,
-                                                                                         const int32_t flags) {
-#if !TSDF_APPLY_REG
-    // per warp: the brick's grid words and accumulators, and the offsets of
-    // its touched voxels (compacted)
-    __shared__ uint32_t s_grid[kRegApplyWarps][kBrickVoxels];
-    __shared__ unsigned long long s_acc[kRegApplyWarps][kBrickVoxels];
-    __shared__ uint16_t s_off[kRegApplyWarps][kBrickVoxels];
-#endif
-    __shared__ unsigned long long red_u[kRegApplyWarps], red_h[kRegApplyWarps];
-    __shared__ unsigned s_last;
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned w = threadIdx.x >> 5;
-    const unsigned gwarp = blockIdx.x * kRegApplyWarps + w;
-    const unsigned nwarps = gridDim.x * kRegApplyWarps;
-    pdl_trigger();
-    pdl_wait();   // list and accumulators come from the earlier kernels
-    // coherent load after the wait (see contrib_kernel), one per CTA
-    if (threadIdx.x == 0) s_last = __ldcg(&m.ctr->brick_count);
+// ---- apply of the plain path: one CTA per SM.
+//
+// FLAGS (windows of at most kFlagBricks bricks): every CTA reads ALL brick
+// flags (64 KB for 512x512x128 voxels, from L2), ranks the touched bricks with
+// one CTA-wide prefix sum and takes every gridDim-th of them, so there is no
+// compaction kernel, no list in memory and no list read before each task. The
+// flags are cleared when all CTAs have read them: the last one to say so has
+// one warp do it while the others work on. Larger windows: the compaction
+// kernel lists the bricks, and each CTA takes every gridDim-th entry.
+//
+// The CTA's bricks are cut into quarter-brick warp tasks. What bounds them is
+// the latency of their loads (1.5 KB a task), so each warp keeps kApplyStages
+// tasks in flight with cp.async into shared memory: at the outdoor scan (4.4 k
+// bricks, 3.6 tasks per warp) that is all of them at once.
+//
+// Counters are published CTA by CTA (see kPubWords): no CTA waits for the
+// others at the end (a fence, a returning atomic and the last CTA's reads were
+// 3 us of every scan).
+//
+// 512 threads and four stages: 1024 threads leave no registers for the next
+// scan's ray set-up beside them (outdoor pass 25.2 us, with four stages), 768
+// threads 23.6, 512 threads 23.1, 384 threads 24.1; fewer than three stages of
+// 512 threads are too little in flight for the corridor (53.9 against 46.2 us).
+// Before (compaction kernel, four CTAs of 128 threads per SM and more, no
+// staging, counters through the last CTA): outdoor 26.8, corridor 51.4, box room
+// 17.9 us a pass; so staged: 23.1, 46.2, 14.4; with the exact quotient of
+// apply_voxel_fast in place of an integer division 22.2, 45.5, 14.3.
+constexpr int kApplyThreads = 512;
+constexpr int kApplyWarpsPlain = kApplyThreads / 32;
+constexpr int kApplyStages = 4;
+constexpr int kApplyPairs = 2;                    // voxel pairs per lane in one task: a quarter brick
+constexpr unsigned kApplyParts = 8u / kApplyPairs;
+constexpr int kStageBytes = 128 * (8 + 4);        // accumulators and grid words of a quarter brick
+constexpr int kApplySmem = kApplyWarpsPlain * kApplyStages * kStageBytes;
+constexpr int kApplyList = 1024;                  // bricks of one CTA listed at a time
+constexpr uint32_t kFlagBricks = 1u << 16;
+constexpr int kFlagVecs = (int)(kFlagBricks / 16) / kApplyThreads;   // 16-flag vectors per thread, at most
+static_assert(kFlagVecs * kApplyThreads * 16 == (int)kFlagBricks && kFlagVecs % 2 == 0, "flags per thread");
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Ranks the bricks whose flags are set and puts the CTA's own (ranks c, c + G,
+// c + 2G, ...) into s_list; returns the number of touched bricks. ginv =
+// ceil(2^32 / G): (rank * ginv) >> 32 is rank / G for rank <= 2^16.
+__device__ __forceinline__ unsigned list_own_bricks(const uint8_t* flag, uint32_t bricks, unsigned c, unsigned G,
+                                                    unsigned ginv, uint32_t* s_list, unsigned* s_warp) {
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint4* fv = reinterpret_cast<const uint4*>(flag);
+    const unsigned nvec = bricks / 16u;   // 0: a window of 1 .. 8 bricks
+    uint4 f[kFlagVecs];
+#pragma unroll
+    for (int j = 0; j < kFlagVecs; ++j) {
+        const unsigned v = (unsigned)j * kApplyThreads + threadIdx.x;
+        f[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (v < nvec) f[j] = __ldcg(fv + v);
+    }
+    if (nvec == 0u && threadIdx.x == 0) {
+        for (uint32_t k = 0; k < bricks; ++k) (k < 4 ? f[0].x : f[0].y) |= (uint32_t)__ldcg(flag + k) << (8u * (k & 3u));
+    }
+    // this thread's touched bricks: a 16-bit mask per vector
+    auto bits4 = [](uint32_t w) { return ((w & 0x01010101u) * 0x01020408u) >> 24 & 0xFu; };   // byte k -> bit k
+    uint32_t mask[kFlagVecs / 2] = {};
+    unsigned cnt = 0;
+#pragma unroll
+    for (int j = 0; j < kFlagVecs; ++j) {
+        if ((f[j].x | f[j].y | f[j].z | f[j].w) == 0u) continue;   // most are empty
+        const uint32_t b = bits4(f[j].x) | bits4(f[j].y) << 4 | bits4(f[j].z) << 8 | bits4(f[j].w) << 12;
+        mask[j / 2] |= b << (16 * (j & 1));
+        cnt += __popc(b);
+    }
+    unsigned incl = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= (unsigned)o) incl += y;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();   // (every thread of the CTA has read its flags)
+    const unsigned t = lane < (unsigned)kApplyWarpsPlain ? s_warp[lane] : 0u;
+    unsigned ti = t;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(kFull, ti, o);
+        if (lane >= (unsigned)o) ti += y;
+    }
+    const unsigned total = __shfl_sync(kFull, ti, 31);
+    const unsigned rank = __shfl_sync(kFull, ti - t, warp) + incl - cnt;   // touched bricks before this thread's
+    if (cnt) {
+        unsigned q = __umulhi(rank, ginv);   // rank / G
+        if (rank - q * G > c) ++q;
+        for (unsigned r = q * G + c; r < rank + cnt; r += G, ++q) {
+            unsigned skip = r - rank;
+            int j = 0;
+            uint32_t b = 0;
+#pragma unroll
+            for (int k = 0; k < kFlagVecs; ++k) {
+                const uint32_t bk = mask[k / 2] >> (16 * (k & 1)) & 0xFFFFu;
+                const unsigned n = __popc(bk);
+                if (b == 0u) {
+                    if (skip < n) {
+                        b = bk;
+                        j = k;
+                    } else {
+                        skip -= n;
+                    }
+                }
+            }
+            for (; skip; --skip) b &= b - 1u;
+            s_list[q] = ((unsigned)j * kApplyThreads + threadIdx.x) * 16u + (unsigned)(__ffs(b) - 1);
+        }
+    }
     __syncthreads();
-    const unsigned nb = s_last;
-    __syncthreads();   // s_last is reused by finish_if_last
+    return total;
+}
+
+template <int MODE, bool FLAGS>
+__global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m, const uint32_t bricks,
+                                                                const unsigned ginv, const int32_t w_max,
+                                                                const int32_t flags) {
+    extern __shared__ __align__(16) unsigned char stages[];
+    __shared__ uint32_t s_list[kApplyList];
+    __shared__ unsigned s_warp[kApplyWarpsPlain];
+    __shared__ unsigned long long red_u[kApplyWarpsPlain], red_h[kApplyWarpsPlain];
+    const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const unsigned G = gridDim.x, c = blockIdx.x;
+    pdl_wait();      // flags or list, and accumulators, come from the earlier kernels
+    pdl_trigger();   // (after the wait: the next scan's ray set-up writes the ray list)
+    unsigned nb;
+    if (FLAGS) {
+        nb = list_own_bricks(m.brick_flag, bricks, c, G, ginv, s_list, s_warp);
+    } else {
+        if (threadIdx.x == 0) s_warp[0] = __ldcg(&m.ctr->brick_count);
+        __syncthreads();
+        nb = s_warp[0];
+    }
+    long long* pub = m.host_last ? m.host_last : m.ctr->pub;
+    if (warp == kApplyWarpsPlain - 1) {
+        unsigned last = 0;
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(&m.ctr->flags_read, 1u) == G - 1u ? 1u : 0u;
+            __threadfence();
+        }
+        if (__shfl_sync(kFull, last, 0)) {   // all CTAs have read the flags (the list's length): clear them
+            if (!FLAGS) {
+                if (lane == 0) m.ctr->brick_count = 0u;
+            } else if (bricks < 16u) {
+                if (lane < bricks) m.brick_flag[lane] = 0;
+            } else {
+                for (unsigned v = lane; v < bricks / 16u; v += 32u)
+                    reinterpret_cast<uint4*>(m.brick_flag)[v] = make_uint4(0u, 0u, 0u, 0u);
+            }
+            if (lane == 0) m.ctr->flags_read = 0u;
+        }
+    } else if (warp == kApplyWarpsPlain - 2 && c == 0u) {
+        // the scan's own counters: valid rays, and in MIN_ABS mode the
+        // contributions that the march counted; both start the next scan at 0
+        LiveCounts* lc = &m.ctr->live[m.parity];
+        unsigned long long h = 0;
+        if (MODE == 1) {
+            h = __ldcg(&m.ctr->part[lane].hits);
+            m.ctr->part[lane].hits = 0ull;
+            for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(kFull, h, o);
+        }
+        if (lane == 0) {
+            pub[0] = (long long)__ldcg(&lc->valid);
+            pub[1] = (long long)h;
+            pub[2] = 0;
+            pub[3] = 0;
+            pub[4] = (long long)G;
+            lc->front = lc->back = lc->valid = 0u;
+        }
+    }
+    // ---- warp tasks: quarters of the CTA's bricks, kApplyStages in flight
+    const unsigned mine = c < nb ? (nb - c + G - 1u) / G : 0u;
+    unsigned char* const ring = stages + (size_t)warp * (kApplyStages * kStageBytes);
     unsigned long long touched = 0, hits = 0;
-#if TSDF_APPLY_REG
-    for (unsigned t = gwarp; t < nb * (8u / kApplyPairs); t += nwarps)
-        apply_part_reg<MODE, kApplyPairs>(m, w_max, flags, t, touched, hits);
-#else
-    for (unsigned i = gwarp; i < nb; i += nwarps)
-        apply_brick<MODE>(m, w_max, flags, i, s_grid[w], s_acc[w], s_off[w], touched, hits);
-#endif
+    for (unsigned b0 = 0; b0 < mine; b0 += kApplyList) {   // CTA-uniform; one round unless a list is very long
+        const unsigned nl = min(mine - b0, (unsigned)kApplyList);
+        if (!FLAGS) {
+            __syncthreads();
+            for (unsigned i = threadIdx.x; i < nl; i += kApplyThreads)
+                s_list[i] = __ldcg(m.brick_list + c + (size_t)(b0 + i) * G);
+            __syncthreads();
+        }
+        const unsigned ntask = nl * kApplyParts;
+        auto fetch = [&](unsigned t, unsigned stage) {
+            if (t < ntask) {
+                const size_t v = ((size_t)s_list[t / kApplyParts] << 9) + (t % kApplyParts) * 128u;
+                ulonglong2* sa = reinterpret_cast<ulonglong2*>(ring + stage * kStageBytes);
+                uint2* sg = reinterpret_cast<uint2*>(ring + stage * kStageBytes + 1024);
+                const ulonglong2* ga = reinterpret_cast<const ulonglong2*>(m.acc + v);
+                const uint2* gg = reinterpret_cast<const uint2*>(m.grid + v);
+                cp_async16(sa + lane, ga + lane);
+                cp_async16(sa + 32 + lane, ga + 32 + lane);
+                cp_async8(sg + lane, gg + lane);
+                cp_async8(sg + 32 + lane, gg + 32 + lane);
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (unsigned k = 0; k < kApplyStages; ++k) fetch(warp + k * kApplyWarpsPlain, k);
+        unsigned stage = 0;
+        for (unsigned t = warp; t < ntask; t += kApplyWarpsPlain) {   // warp-uniform
+            cp_async_wait<kApplyStages - 1>();   // (a lane reads only what it copied itself)
+            const size_t v = ((size_t)s_list[t / kApplyParts] << 9) + (t % kApplyParts) * 128u;
+            const ulonglong2* sa = reinterpret_cast<const ulonglong2*>(ring + stage * kStageBytes);
+            const uint2* sg = reinterpret_cast<const uint2*>(ring + stage * kStageBytes + 1024);
+            ulonglong2 acc[kApplyPairs] = {sa[lane], sa[32 + lane]};
+            uint2 g[kApplyPairs] = {sg[lane], sg[32 + lane]};
+            apply_pairs<MODE, kApplyPairs>(w_max, flags, acc, g, sg, touched, hits);
+            fetch(t + kApplyStages * kApplyWarpsPlain, stage);
+            store_pairs<kApplyPairs>(reinterpret_cast<uint2*>(m.grid + v), reinterpret_cast<ulonglong2*>(m.acc + v), acc, g);
+            stage = stage + 1u == kApplyStages ? 0u : stage + 1u;
+        }
+        cp_async_wait<0>();
+    }
     for (int o = 16; o > 0; o >>= 1) {
         touched += __shfl_xor_sync(kFull, touched, o);
         hits += __shfl_xor_sync(kFull, hits, o);
     }
     if (lane == 0) {
-        red_u[w] = touched;
-        red_h[w] = hits;
+        red_u[warp] = touched;
+        red_h[warp] = hits;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long bu = 0, bh = 0;
-        for (int k = 0; k < kRegApplyWarps; ++k) {
-            bu += red_u[k];
-            bh += red_h[k];
+    if (warp == 0) {
+        touched = lane < (unsigned)kApplyWarpsPlain ? red_u[lane] : 0ull;
+        hits = lane < (unsigned)kApplyWarpsPlain ? red_h[lane] : 0ull;
+        for (int o = 16; o > 0; o >>= 1) {
+            touched += __shfl_xor_sync(kFull, touched, o);
+            hits += __shfl_xor_sync(kFull, hits, o);
         }
-        if (bu) atomicAdd(&m.ctr->part[blockIdx.x % kParts].touched, bu);
-        if (MODE == 0 && bh) atomicAdd(&m.ctr->part[blockIdx.x % kParts].hits, bh);
+        // (in MIN_ABS mode the contributions are the march's count)
+        if (lane == 0) *reinterpret_cast<longlong2*>(pub + 8 + 2 * c) = make_longlong2((long long)touched, MODE == 0 ? (long long)hits : 0);
     }
-    finish_if_last(m, &s_last);
 }
 
 // Sort reduction: one warp per listed brick (as apply_kernel, and likewise
@@ -509,8 +677,8 @@ __global__ void __launch_bounds__(kApplyWarps * 32) sort_apply_kernel(const MapD
     const unsigned w = threadIdx.x >> 5;
     const unsigned gwarp = blockIdx.x * kApplyWarps + w;
     const unsigned nwarps = gridDim.x * kApplyWarps;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();   // (after the wait: the next scan's ray set-up writes the ray list)
     unsigned nb = 0, ovf = 0;
     if (lane == 0) {
         nb = __ldcg(&m.ctr->brick_count);
@@ -556,8 +724,8 @@ __global__ void __launch_bounds__(kApplyWarps * 32) pool_apply_kernel(const MapD
     const unsigned w = threadIdx.x >> 5;
     const unsigned gwarp = blockIdx.x * kApplyWarps + w;
     const unsigned nwarps = gridDim.x * kApplyWarps;
-    pdl_trigger();
     pdl_wait();
+    pdl_trigger();   // (after the wait: the next scan's ray set-up writes the ray list)
     unsigned ns = 0, ovf = 0;
     if (lane == 0) {
         ns = __ldcg(&m.ctr->pool_count);
@@ -600,13 +768,15 @@ __global__ void __launch_bounds__(kApplyWarps * 32) pool_apply_kernel(const MapD
     finish_if_last(m, &s_last);
 }
 
-// Launch with programmatic stream serialisation when `pdl` is set.
+// Launch with `smem` bytes of dynamic shared memory, with programmatic stream
+// serialisation when `pdl` is set.
 template <typename... KArgs, typename... Args>
-cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, bool pdl, Args&&... args) {
+cudaError_t launch_smem(size_t smem, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, bool pdl,
+                        Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -614,6 +784,26 @@ cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t s, bool pdl, Args&&... args) {
+    return launch_smem(0, kernel, grid, block, s, pdl, std::forward<Args>(args)...);
+}
+
+// Allows `kernel` `bytes` of dynamic shared memory on the current device (once
+// per kernel and device).
+cudaError_t allow_smem(const void* kernel, int bytes) {
+    static std::mutex mu;
+    static std::set<std::pair<const void*, int>> done;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    if (done.count({kernel, dev})) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.insert({kernel, dev});
+    return e;
 }
 
 // CTAs of `kernel` (launched with `threads` threads and static shared memory
@@ -790,7 +980,7 @@ cudaError_t launch_sort_scatter(const MapDev& m, bool pdl, cudaStream_t s) {
 cudaError_t launch_sort_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
                               cudaStream_t s) {
     auto* k = reduce == 0 ? sort_apply_kernel<0> : sort_apply_kernel<1>;
-    return launch(k, resident_grid(k, kApplyWarps * 32, TSDF_APPLY_CTAS_PER_SM), dim3(kApplyWarps * 32), s, pdl, m,
+    return launch(k, resident_grid(k, kApplyWarps * 32), dim3(kApplyWarps * 32), s, pdl, m,
                   w_max, flags);
 }
 
@@ -799,10 +989,21 @@ cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStrea
     return launch(compact_kernel, dim3((nwords + 255u) / 256u), dim3(256), s, pdl, m, nwords);
 }
 
-cudaError_t launch_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl, cudaStream_t s) {
-    auto* k = reduce == 0 ? apply_kernel<0> : apply_kernel<1>;
-    return launch(k, resident_grid(k, kRegApplyWarps * 32, TSDF_APPLY_CTAS_PER_SM), dim3(kRegApplyWarps * 32), s,
-                  pdl, m, w_max, flags);
+cudaError_t launch_apply(const MapDev& m, uint32_t bricks, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
+                         cudaStream_t s) {
+    const unsigned sms = resident_grid(apply_kernel<0, true>, kApplyThreads, 1).x;
+    const unsigned G = std::min(sms, (unsigned)kMaxApplyCtas);
+    const bool by_flags = bricks <= kFlagBricks && (bricks + G - 1) / G <= (uint32_t)kApplyList;
+    if (!by_flags) {
+        const cudaError_t e = launch_compact(m, bricks, pdl, s);
+        if (e != cudaSuccess) return e;
+    }
+    auto* k = by_flags ? (reduce == 0 ? apply_kernel<0, true> : apply_kernel<1, true>)
+                       : (reduce == 0 ? apply_kernel<0, false> : apply_kernel<1, false>);
+    const cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), kApplySmem);
+    if (e != cudaSuccess) return e;
+    const unsigned ginv = (unsigned)(((1ull << 32) + G - 1) / G);
+    return launch_smem(kApplySmem, k, dim3(G), dim3(kApplyThreads), s, pdl, m, bricks, ginv, w_max, flags);
 }
 
 }  // namespace tsdf

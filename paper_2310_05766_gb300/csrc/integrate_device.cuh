@@ -148,19 +148,14 @@ __device__ __forceinline__ void ray_setup(const ScanArgs& a, float4 p, bool in, 
     }
 }
 
-// ---- rays: the CTA's 32 NW threads set up points [base, base + 32 NW) of a
-// scan and append the live ones to the map's ray list. With SORT each live ray also
-// reserves its pair slots (one 64-bit atomic per CTA). With SPLIT the rays
-// whose fill reaches at least one voxel each side at the hit (delta_z r >= vs,
-// the costly ones) go to the front of the list and the others to its end
-// (entry ray_cap - 1 - j for the j-th), so that the contribution kernel can
-// take the costly work first; with both ends counted, they never meet. With
+// ---- rays, sort reduction: the CTA's 32 NW threads set up points [base,
+// base + 32 NW) of a scan, append the live ones to the map's ray list and
+// reserve their pair slots (one 32-bit and one 64-bit atomic per CTA). With
 // PDL the wait for the preceding grid comes before the first access to the
 // map's counters and ray list.
-template <bool PDL, bool SORT, bool SPLIT = false, int NW = 8>
-__device__ __forceinline__ void rays_task(const ScanArgs& a, const MapDev& m, int base, unsigned part,
-                                          RaysSmemT<NW>* sm) {
-    static_assert(!(SORT && SPLIT), "the sort reduction keeps one list");
+template <bool PDL, int NW>
+__device__ __forceinline__ void rays_task_sort(const ScanArgs& a, const MapDev& m, int base, unsigned part,
+                                               RaysSmemT<NW>* sm) {
     const int i = base + (int)threadIdx.x;
     const unsigned lane = threadIdx.x & 31u;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -170,71 +165,50 @@ __device__ __forceinline__ void rays_task(const ScanArgs& a, const MapDev& m, in
     float4 ra, rb;
     bool valid, live;
     ray_setup(a, p, in, ra, rb, valid, live);
-    // pair slots of this ray (sort reduction): an inclusive warp scan
-    uint32_t nslot = 0, sincl = 0;
-    if (SORT) {
-        nslot = live ? ray_slots(a, ra.w, rb.w != 0.f) : 0u;
-        const uint32_t own = nslot == kNoSlot ? 0u : nslot;
-        sincl = own;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, sincl, o);
-            if (lane >= (unsigned)o) sincl += y;
-        }
+    // pair slots of this ray: an inclusive warp scan
+    const uint32_t nslot = live ? ray_slots(a, ra.w, rb.w != 0.f) : 0u;
+    const uint32_t own = nslot == kNoSlot ? 0u : nslot;
+    uint32_t sincl = own;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, sincl, o);
+        if (lane >= (unsigned)o) sincl += y;
     }
-    // CTA-level compaction of the live rays: one list atomic per CTA (per end)
+    // CTA-level compaction of the live rays: one list atomic per CTA
     const unsigned warp = threadIdx.x >> 5;
-    const bool heavy = !SPLIT || (live && rb.w != 0.f && fm(fm(a.dz, ra.w), a.inv_vs) >= 1.f);
-    const unsigned lmask = __ballot_sync(kFull, live && heavy);
-    const unsigned bmask = SPLIT ? __ballot_sync(kFull, live && !heavy) : 0u;
+    const unsigned lmask = __ballot_sync(kFull, live);
     const unsigned vmask = __ballot_sync(kFull, valid);
     if (lane == 0) {
         sm->wl[warp] = __popc(lmask);
         sm->wv[warp] = __popc(vmask);
-        if (SPLIT) sm->wb[warp] = __popc(bmask);
     }
-    if (SORT && lane == 31) sm->ws[warp] = sincl;
+    if (lane == 31) sm->ws[warp] = sincl;
     __syncthreads();
-    if (PDL) pdl_wait();   // the previous scan's finish kernel resets live_count and the counters
+    if (PDL) pdl_wait();   // the previous scan's finish resets live_count and the counters
     if (threadIdx.x == 0) {
-        unsigned tl = 0, tv = 0, tb = 0, ts32 = 0;
+        unsigned tl = 0, tv = 0, ts32 = 0;
         unsigned long long ts = 0;
         for (int w = 0; w < NW; ++w) {
-            const unsigned l = sm->wl[w], b = SPLIT ? sm->wb[w] : 0u, q = SORT ? sm->ws[w] : 0u;
+            const unsigned l = sm->wl[w], q = sm->ws[w];
             sm->wl[w] = tl;
             tl += l;
             tv += sm->wv[w];
-            if (SPLIT) {
-                sm->wb[w] = tb;
-                tb += b;
-            }
-            if (SORT) {
-                sm->ws[w] = ts32;
-                ts32 += q;
-                ts += q;
-            }
+            sm->ws[w] = ts32;
+            ts32 += q;
+            ts += q;
         }
         sm->base = tl ? atomicAdd(&m.ctr->live_count, tl) : 0u;
-        if (SPLIT) sm->bbase = tb ? atomicAdd(&m.ctr->live_back, tb) : 0u;
         if (tv) atomicAdd(&m.ctr->part[part % kParts].valid, (unsigned long long)tv);
-        if (SORT) sm->sbase = ts ? atomicAdd(&m.ctr->slot_count, ts) : 0ull;
+        sm->sbase = ts ? atomicAdd(&m.ctr->slot_count, ts) : 0ull;
     }
     __syncthreads();
     if (live) {
-        const unsigned below = (1u << lane) - 1u;
-        unsigned off;
-        if (heavy) {
-            off = sm->base + sm->wl[warp] + __popc(lmask & below);
-        } else {
-            off = m.ray_cap - 1u - (sm->bbase + sm->wb[warp] + __popc(bmask & below));
-        }
+        const unsigned off = sm->base + sm->wl[warp] + __popc(lmask & ((1u << lane) - 1u));
         m.ray_a[off] = ra;
         m.ray_b[off] = rb;
-        if (SORT) {
-            const unsigned long long first = sm->sbase + sm->ws[warp] + (sincl - (nslot == kNoSlot ? 0u : nslot));
-            // slots at or beyond the capacity overflow, sample by sample
-            m.ray_slot[off] = nslot == kNoSlot ? kNoSlot
-                                                : (uint32_t)(first < m.pair_cap ? first : (unsigned long long)m.pair_cap);
-        }
+        const unsigned long long first = sm->sbase + sm->ws[warp] + (sincl - own);
+        // slots at or beyond the capacity overflow, sample by sample
+        m.ray_slot[off] = nslot == kNoSlot ? kNoSlot
+                                            : (uint32_t)(first < m.pair_cap ? first : (unsigned long long)m.pair_cap);
     }
 }
 
@@ -258,8 +232,18 @@ constexpr int kBatchRaysPPT = TSDF_BATCH_RAYS_PPT;
 // CTA's threads set up points [base, base + 32 NW PPT), thread t the points
 // base + PPT t .. base + PPT t + PPT - 1, whose loads are all in flight at
 // once, and append the live ones (in point order) to the map's ray list with
-// one list atomic per CTA and list end, as rays_task does for one point per
-// thread. Same rays, same per-ray results; only fewer CTAs and atomics.
+// one list atomic per CTA and list end.
+// SPLIT (the per-map plain path): the rays whose fill reaches at least one
+// voxel each side at the hit (delta_z r >= vs, the costly ones) go to the
+// front of the list and the others to its end (entry ray_cap - 1 - j for the
+// j-th), so that the contribution kernel can take the costly work first; with
+// both ends counted, they never meet. Its counts are the scan's own (LiveCounts
+// by parity) and its list was last read by the previous scan's contributions,
+// which are over when this kernel starts (every apply kernel triggers its
+// dependents after its own wait): so nothing here waits for the previous scan,
+// and the set-up runs beside its apply (the kernel's first CTA waits before it
+// ends, so that what follows sees that scan complete).
+// Otherwise, with PDL, the wait comes before the map's counters and ray list.
 template <bool PDL, bool SPLIT, int NW, int PPT>
 __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m, int base, unsigned part,
                                               RaysSmemT<NW>* sm) {
@@ -303,7 +287,7 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
         sm->wv[warp] = wv;
     }
     __syncthreads();
-    if (PDL) pdl_wait();   // the previous scan's finish kernel resets live_count and the counters
+    if (PDL && !SPLIT) pdl_wait();   // the previous scan's finish resets live_count and the counters
     if (threadIdx.x == 0) {
         unsigned tl = 0, tv = 0, tb = 0;
         for (int w = 0; w < NW; ++w) {
@@ -314,9 +298,15 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
             tb += b;
             tv += sm->wv[w];
         }
-        sm->base = tl ? atomicAdd(&m.ctr->live_count, tl) : 0u;
-        sm->bbase = SPLIT && tb ? atomicAdd(&m.ctr->live_back, tb) : 0u;
-        if (tv) atomicAdd(&m.ctr->part[part % kParts].valid, (unsigned long long)tv);
+        if (SPLIT) {
+            LiveCounts* lc = &m.ctr->live[m.parity];
+            sm->base = tl ? atomicAdd(&lc->front, tl) : 0u;
+            sm->bbase = tb ? atomicAdd(&lc->back, tb) : 0u;
+            if (tv) atomicAdd(&lc->valid, tv);
+        } else {
+            sm->base = tl ? atomicAdd(&m.ctr->live_count, tl) : 0u;
+            if (tv) atomicAdd(&m.ctr->part[part % kParts].valid, (unsigned long long)tv);
+        }
     }
     __syncthreads();
     unsigned off_l = sm->base + sm->wl[warp] + il - cl;     // first front entry of this thread
@@ -333,6 +323,7 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
             ++off_b;
         }
     }
+    if (PDL && SPLIT && blockIdx.x == 0) pdl_wait();
 }
 
 // ---- contrib: rays of one 32-ray block (one per lane, dead lanes r = -1);
@@ -825,12 +816,119 @@ __device__ __forceinline__ void apply_staged(const MapDev& m, int32_t w_max, int
     for (int v = 0; v < 4; ++v) gpw[32 * v + lane] = sg4[32 * v + lane];
 }
 
-// ---- apply, register form: one warp updates grid brick `brick` from the 512
-// accumulators at `accp` (a brick of the dense accumulator or a pool slot).
-// Lane l holds voxels 2(32 v + l) and +1 (v = 0..7) as eight 8-byte grid pairs
-// and eight 16-byte accumulator pairs, all loaded at once; every touched voxel
-// is decoded in place (16 independent updates per lane), and only changed
-// pairs are written back and reset.
+// Eq. 1 / Eq. 2 of one voxel without branches, for the usual case of
+// decode_apply: a 32-bit sum, a count below 2^15, a non-negative weight; any
+// other sets bits of `wide` (the caller then takes decode_apply). An untouched
+// voxel keeps its word.
+//
+// The rounded quotient (half away from zero) is estimated as the nearest
+// integer to num times an approximate reciprocal of den, taken 2^-19 too small,
+// and made exact with the integer remainder: |num| / den <= 32768 (a weighted
+// mean of 16-bit codes), and the conversion of num (2^-24), rcp.approx (2^-23)
+// and the product's roundings are off by less than 2^-21 together, so the
+// estimate is never beyond the exact result and less than one short of it: one
+// step away from zero, when twice the remainder reaches den, corrects it.
+// (The integer pipe bounds the apply, so the products and the rounding run on
+// the other pipes: 320 -> 180 instructions per task of four voxels a lane.)
+template <int MODE>
+__device__ __forceinline__ void apply_voxel_fast(unsigned long long P, uint32_t& word, int32_t w_max, unsigned& wide,
+                                                 unsigned& touched, unsigned& hits) {
+    const unsigned lo = (unsigned)P, hi = (unsigned)(P >> 32);
+    int S;
+    unsigned W;
+    if (MODE == 0) {
+        const unsigned t = hi + (lo >> 31);   // count in bits 8.., low byte 0 when the sum fits 32 bits
+        S = (int)lo;
+        W = t >> 8;
+        wide |= (t & 0xFF8000FFu) | (((lo + 0x40000000u) | word) & 0x80000000u);
+    } else {
+        const unsigned key = 65536u - lo;
+        const int mag = (int)(key >> 1);
+        S = (key & 1u) ? -mag : mag;
+        W = lo != 0u ? 1u : 0u;
+        wide |= word & 0x80000000u;
+    }
+    const int gv = (int)(int16_t)(word & 0xFFFFu);
+    const int gw = (int)word >> 16;
+    const int num = gv * gw + S;
+    const int den = gw + (int)W;
+    float rc;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(__int2float_rn(den)));
+    rc = fm(rc, 1.0f - 0x1p-19f);
+    int q = __float_as_int(__fmaf_rn(__int2float_rn(num), rc, 12582912.0f)) - 0x4B400000;
+    const int rem = num - q * den;
+    if (2 * abs(rem) >= den) q += (num >> 31) | 1;
+    const int nw = min(den, w_max);
+    if (W != 0u) {
+        word = __byte_perm((unsigned)q, (unsigned)nw, 0x5410);
+        ++touched;
+    }
+    hits += W;
+}
+
+// A voxel by the general path; rare, so out of line.
+template <int MODE>
+static __device__ __noinline__ uint32_t apply_voxel_wide(unsigned long long P, uint32_t word, int32_t w_max,
+                                                         int32_t flags) {
+    decode_apply<MODE>(P, word, w_max, flags);
+    return word;
+}
+
+// Contributions of an accumulator (MIN_ABS: 1 for a touched voxel).
+template <int MODE>
+__device__ __forceinline__ unsigned contributions(unsigned long long P) {
+    const long long S = ((long long)(P << 24)) >> 24;
+    return MODE == 0 ? (unsigned)((P - (unsigned long long)S) >> 40) : (P != 0ull ? 1u : 0u);
+}
+
+// The voxels of a lane's NV pairs: accumulators acc, grid words g (updated),
+// read from gsrc (where they still are).
+template <int MODE, int NV>
+__device__ __forceinline__ void apply_pairs(int32_t w_max, int32_t flags, const ulonglong2 (&acc)[NV], uint2 (&g)[NV],
+                                            const uint2* gsrc, unsigned long long& touched, unsigned long long& hits) {
+    const unsigned lane = threadIdx.x & 31u;
+    unsigned cnt = 0, h = 0, wide = MODE == 0 ? (unsigned)(flags & kFlagScanWeight) : 0u;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        // (a row is an 8 x 8 slice of the brick: 28 % of a listed brick's are untouched)
+        if (!__any_sync(kFull, (acc[v].x | acc[v].y) != 0ull)) continue;
+        apply_voxel_fast<MODE>(acc[v].x, g[v].x, w_max, wide, cnt, h);
+        apply_voxel_fast<MODE>(acc[v].y, g[v].y, w_max, wide, cnt, h);
+    }
+    if (wide) {   // some voxel outside the usual case, or the per-scan weight reading: this lane again
+        cnt = h = 0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            g[v] = gsrc[32 * v + lane];
+            if (acc[v].x != 0ull) g[v].x = apply_voxel_wide<MODE>(acc[v].x, g[v].x, w_max, flags);
+            if (acc[v].y != 0ull) g[v].y = apply_voxel_wide<MODE>(acc[v].y, g[v].y, w_max, flags);
+            cnt += (acc[v].x != 0ull ? 1u : 0u) + (acc[v].y != 0ull ? 1u : 0u);
+            h += contributions<MODE>(acc[v].x) + contributions<MODE>(acc[v].y);
+        }
+    }
+    touched += cnt;
+    hits += h;
+}
+
+// Writes the touched pairs back and resets their accumulators.
+template <int NV>
+__device__ __forceinline__ void store_pairs(uint2* gp, ulonglong2* ap, const ulonglong2 (&acc)[NV],
+                                            const uint2 (&g)[NV]) {
+    const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if ((acc[v].x | acc[v].y) != 0ull) {
+            gp[32 * v + lane] = g[v];
+            ap[32 * v + lane] = make_ulonglong2(0ull, 0ull);
+        }
+    }
+}
+
+// ---- apply, register form (batches and the pool reduction): one warp updates
+// grid brick `brick` from the 512 accumulators at `accp` (a brick of the dense
+// accumulator or a pool slot). Lane l holds voxels 2(32 v + l) and +1 as 8-byte
+// grid pairs and 16-byte accumulator pairs, all loaded at once; every touched
+// voxel is decoded in place, and only changed pairs are written back and reset.
 // NV voxel pairs per lane, starting at pair row v0: NV = 8 is the whole
 // brick, NV = 4 (v0 = 0 or 4) one half, NV = 2 a quarter.
 template <int MODE, int NV = 8>
@@ -838,6 +936,12 @@ __device__ __forceinline__ void apply_brick_at(const MapDev& m, int32_t w_max, i
                                                unsigned long long* accp, unsigned long long& touched,
                                                unsigned long long& hits, unsigned v0 = 0) {
     static_assert(NV == 8 || NV == 4 || NV == 2, "whole, half or quarter bricks");
+    if constexpr (NV == 8) {   // two halves, one after the other: all sixteen voxels at once would not fit the registers
+#pragma unroll 1
+        for (unsigned h = 0; h < 8u; h += 4u)
+            apply_brick_at<MODE, 4>(m, w_max, flags, brick, accp, touched, hits, h);
+        return;
+    }
     const unsigned lane = threadIdx.x & 31u;
     uint2* gp = reinterpret_cast<uint2*>(m.grid + ((size_t)brick << 9)) + 32 * v0;
     ulonglong2* ap = reinterpret_cast<ulonglong2*>(accp) + 32 * v0;
@@ -847,35 +951,8 @@ __device__ __forceinline__ void apply_brick_at(const MapDev& m, int32_t w_max, i
     for (int v = 0; v < NV; ++v) acc[v] = ap[32 * v + lane];
 #pragma unroll
     for (int v = 0; v < NV; ++v) g[v] = gp[32 * v + lane];
-    unsigned cnt = 0;
-    unsigned long long h = 0;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        if (acc[v].x != 0ull) {
-            h += decode_apply<MODE>(acc[v].x, g[v].x, w_max, flags);
-            ++cnt;
-        }
-        if (acc[v].y != 0ull) {
-            h += decode_apply<MODE>(acc[v].y, g[v].y, w_max, flags);
-            ++cnt;
-        }
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        if ((acc[v].x | acc[v].y) != 0ull) {
-            gp[32 * v + lane] = g[v];
-            ap[32 * v + lane] = make_ulonglong2(0ull, 0ull);
-        }
-    }
-    touched += cnt;
-    hits += h;
-}
-
-template <int MODE>
-__device__ __forceinline__ void apply_brick_reg(const MapDev& m, int32_t w_max, int32_t flags, unsigned i,
-                                                unsigned long long& touched, unsigned long long& hits) {
-    const unsigned brick = m.brick_list[i];
-    apply_brick_at<MODE>(m, w_max, flags, brick, m.acc + ((size_t)brick << 9), touched, hits);
+    apply_pairs<MODE, NV>(w_max, flags, acc, g, gp, touched, hits);
+    store_pairs<NV>(gp, ap, acc, g);
 }
 
 // Part t % P of listed brick t / P (P = 8 / NV parts per brick).
@@ -1092,8 +1169,8 @@ __device__ __forceinline__ void sort_apply_brick(const MapDev& m, int32_t w_max,
     __syncwarp();
 }
 
-// ---- finish: one warp (lane = counter slot) publishes the scan's counters
-// and clears the per-scan state.
+// ---- finish (sort and pool reductions, batches): one warp (lane = counter
+// slot) publishes the scan's counters and clears the per-scan state.
 __device__ __forceinline__ void finish_warp(const MapDev& m) {
     MapCounters* c = m.ctr;
     const unsigned lane = threadIdx.x & 31u;
@@ -1112,15 +1189,17 @@ __device__ __forceinline__ void finish_warp(const MapDev& m) {
         // a pool-reduction scan that found the pool full was dropped
         const long long st = __ldcg(&c->pool_overflow) != 0u ? kStatusCapacity : 0;
         if (st != 0) h = u = 0ull;
-        c->last_valid = (long long)v;
-        c->last_hits = (long long)h;
-        c->last_touched = (long long)u;
-        c->last_status = st;
+        c->pub[0] = (long long)v;
+        c->pub[1] = (long long)h;
+        c->pub[2] = (long long)u;
+        c->pub[3] = st;
+        c->pub[4] = 0;
         if (m.host_last) {   // also into host memory: reading them needs no copy
             m.host_last[0] = (long long)v;
             m.host_last[1] = (long long)h;
             m.host_last[2] = (long long)u;
             m.host_last[3] = st;
+            m.host_last[4] = 0;
         }
         c->live_count = 0u;
         c->brick_count = 0u;
@@ -1129,7 +1208,6 @@ __device__ __forceinline__ void finish_warp(const MapDev& m) {
         c->apply_done = 0u;
         c->pool_count = 0u;
         c->pool_overflow = 0u;
-        c->live_back = 0u;
     }
 }
 

@@ -190,13 +190,13 @@ extern "C" int tsdf_integrate_static(uint32_t* grid_dev, const tsdf_params* para
         }
         launched_contrib = true;
     }
-    if (e == cudaSuccess) e = launch_compact(md, (uint32_t)bricks, true, s);
-    if (e == cudaSuccess) e = launch_apply(md, params->reduce, params->w_max, params->flags, true, s);
+    if (e == cudaSuccess) e = launch_apply(md, (uint32_t)bricks, params->reduce, params->w_max, params->flags, true, s);
     if (e == cudaSuccess && stats_host) {
-        long long last[3] = {0, 0, 0};
-        e = cudaMemcpyAsync(last, &md.ctr->last_valid, sizeof(last), cudaMemcpyDeviceToHost, s);
+        long long pub[kPubWords] = {}, last[3] = {0, 0, 0};
+        e = cudaMemcpyAsync(pub, md.ctr->pub, sizeof(pub), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e == cudaSuccess) {
+            sum_counters(pub, last);
             stats_host->valid_rays = last[0];
             stats_host->hits = last[1];
             stats_host->touched = last[2];

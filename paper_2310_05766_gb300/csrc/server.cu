@@ -71,7 +71,7 @@ struct Slot {
     cudaStream_t stream = nullptr;
     tsdf_batch* batch = nullptr;
     float4* dev_pts = nullptr;          // max_batch x max_points
-    long long* counters = nullptr;      // pinned, max_batch x 3 (maps without mapped counters)
+    long long* counters = nullptr;      // pinned, max_batch x kPubWords (maps without mapped counters)
     cudaEvent_t done = nullptr;
     std::vector<Request*> reqs;
     std::vector<const volatile long long*> src;   // per request: where its counters are read
@@ -181,9 +181,10 @@ int launch_batch(tsdf_server* s, int k, std::vector<Request*>& reqs, const std::
     for (int i = 0; i < count && e == cudaSuccess; ++i) {
         sl.src[i] = map_host_counters(maps[i]);
         if (!sl.src[i]) {
-            e = cudaMemcpyAsync(sl.counters + 3 * i, map_last_counters(maps[i]), 3 * sizeof(long long),
-                                cudaMemcpyDeviceToHost, sl.stream);
-            sl.src[i] = sl.counters + 3 * i;
+            long long* dst = sl.counters + (size_t)kPubWords * i;
+            e = cudaMemcpyAsync(dst, map_last_counters(maps[i]), kPubWords * sizeof(long long), cudaMemcpyDeviceToHost,
+                                sl.stream);
+            sl.src[i] = dst;
         }
     }
     if (e == cudaSuccess) e = cudaEventRecord(sl.done, sl.stream);
@@ -216,9 +217,11 @@ void worker_loop(tsdf_server* s) {
             const double t = now_us();
             for (size_t i = 0; i < sl.reqs.size(); ++i) {
                 Request* r = sl.reqs[i];
-                r->res.stats.valid_rays = sl.src[i][0];
-                r->res.stats.hits = sl.src[i][1];
-                r->res.stats.touched = sl.src[i][2];
+                long long last[3];
+                sum_counters(sl.src[i], last);
+                r->res.stats.valid_rays = last[0];
+                r->res.stats.hits = last[1];
+                r->res.stats.touched = last[2];
                 r->res.t_done_us = t;
                 r->res.batch_size = (int32_t)sl.reqs.size();
                 r->res.status = TSDF_OK;
@@ -328,7 +331,7 @@ int tsdf_server_create(const tsdf_server_config* cfg, tsdf_server** out) {
     for (Slot& sl : s->slots) {
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaMalloc(&sl.dev_pts, (size_t)cfg->max_batch * cfg->max_points * sizeof(float4));
-        if (e == cudaSuccess) e = cudaMallocHost(&sl.counters, (size_t)cfg->max_batch * 3 * sizeof(long long));
+        if (e == cudaSuccess) e = cudaMallocHost(&sl.counters, (size_t)cfg->max_batch * kPubWords * sizeof(long long));
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
         if (e != cudaSuccess) break;
         int rc = tsdf_batch_create(cfg->max_batch, &sl.batch);

@@ -26,12 +26,29 @@ struct CounterPart {
     unsigned long long touched;     // voxels updated
     unsigned long long pad[13];
 };
+
+// Published counters of the last completed scan, in device memory and, when
+// the map has it, mapped host memory: words 0..3 are valid rays, contributions,
+// touched voxels and status (0, or TSDF_ERR_CAPACITY when the scan was dropped:
+// pool full); word 4 is the number of CTAs whose own (touched voxels,
+// contributions) follow from word 8 on and are still to be added
+// (sum_counters): the plain path's apply publishes them CTA by CTA, so that no
+// CTA waits for another.
+constexpr int kMaxApplyCtas = 160;
+constexpr int kPubWords = 8 + 2 * kMaxApplyCtas;
+
+// Rays of a plain scan (split ray list): heavy ones from the list's front,
+// light ones from its end, and valid points. Two of them, used in turn by
+// consecutive scans (MapDev::parity): the ray set-up counts into one while the
+// previous scan's apply still reads and clears the other.
+struct LiveCounts {
+    unsigned int front, back, valid, pad;
+};
+
 struct MapCounters {
     CounterPart part[kParts];
-    long long last_valid;           // counters of the last completed scan
-    long long last_hits;
-    long long last_touched;
-    long long last_status;          // 0, or TSDF_ERR_CAPACITY when the scan was dropped (pool full)
+    long long pub[kPubWords];
+    LiveCounts live[2];
     unsigned int live_count;        // rays of the scan in flight that can reach the window (compacted)
     unsigned int brick_count;       // length of the touched-brick list of the scan in flight
     unsigned long long slot_count;  // sort reduction: pair slots reserved by the scan in flight
@@ -40,7 +57,7 @@ struct MapCounters {
     unsigned long long surface_count;   // points found by the last surface extraction
     unsigned int pool_count;        // pool reduction: slots claimed by the scan in flight (may exceed the capacity)
     unsigned int pool_overflow;     // pool reduction: 1 if a brick found the pool full (the scan is dropped)
-    unsigned int live_back;         // split ray list: light rays of the scan in flight, stored from the list's end
+    unsigned int flags_read;        // CTAs of the plain apply that have read the brick flags or the list length
     unsigned int pad_;
 };
 
@@ -63,7 +80,9 @@ struct MapDev {
     float4* ray_b;                  // per live ray (compacted): (int.x, int.y, int.z, fill ? 1 : 0)
     uint32_t ray_cap;               // entries of ray_a / ray_b (the split list fills them from both ends)
     MapCounters* ctr;
-    long long* host_last;           // mapped pinned host copy of last_valid / hits / touched / status, or null
+    long long* host_last;           // mapped pinned host memory for the published counters (kPubWords), or null
+    uint32_t parity;                // which LiveCounts the plain scan in flight uses
+    uint32_t pad_;
     // sort reduction (null / 0 when the map has no sort buffers)
     uint32_t* brick_slot;           // per brick: its position in the brick list (touched bricks only)
     uint32_t* seg_count;            // per list position: pair count, then the scatter cursor; zero between scans
@@ -164,12 +183,22 @@ struct BatchItem {
 // `map`, grow its ray buffers if needed and fill the batch item.
 int prepare_batch_item(::tsdf_map* map, const float* points_dev, int64_t n, const float pose[12], BatchItem* out);
 int map_device(const ::tsdf_map* map);
-// Device address of the map's published counters (last_valid, last_hits,
-// last_touched: three contiguous int64).
+// Device address of the map's published counters (kPubWords words).
 const long long* map_last_counters(const ::tsdf_map* map);
-// Host address of the mapped pinned copy of those counters, which the last CTA
-// of every integration (per-map or batched) writes; null when the map has none.
+// Host address of the mapped pinned copy of those counters, which every
+// integration (per-map or batched) writes; null when the map has none.
 const volatile long long* map_host_counters(const ::tsdf_map* map);
+// Valid rays, contributions and touched voxels from published counters.
+inline void sum_counters(const volatile long long* pub, long long out[3]) {
+    out[0] = pub[0];
+    out[1] = pub[1];
+    out[2] = pub[2];
+    const long long n = pub[4];
+    for (long long c = 0; c < n; ++c) {
+        out[2] += pub[8 + 2 * c];
+        out[1] += pub[8 + 2 * c + 1];
+    }
+}
 // Grow the map's per-ray buffers to hold n points (synchronous allocation).
 int map_reserve_points(::tsdf_map* map, int64_t n);
 
@@ -204,7 +233,10 @@ cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool
 cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
                            cudaStream_t s);
 cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStream_t s);
-cudaError_t launch_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl, cudaStream_t s);
+// Eq. 1 / Eq. 2 on the bricks whose flags are set (and the flags' reset, and
+// the scan's counters).
+cudaError_t launch_apply(const MapDev& m, uint32_t bricks, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
+                         cudaStream_t s);
 // Sort reduction: emit pairs, count per brick, prefix, scatter, reduce + apply.
 cudaError_t launch_emit(const ScanArgs& a, const MapDev& m, int32_t reduce, int kpt, bool pdl, cudaStream_t s);
 cudaError_t launch_sort_count(const MapDev& m, bool pdl, cudaStream_t s);

@@ -38,3 +38,20 @@ def test_long_marches_exact(n, tau, reduce):
     pose = synth.pose12(synth.rot_zyx(-0.3, 0.05, 0.1), np.array([0.02, 0.1, -0.05]))
     steps = [("scan", _points(n, 5 * n, 0.5, 2.5), pose)] * 2
     assert_same(run_gpu(p, steps, torch), run_oracle(p, steps), f"n={n} tau={tau}")
+
+
+@pytest.mark.parametrize("reduce,flags", [(0, 0), (0, 2), (1, 0)])
+@pytest.mark.parametrize("w_max", [1, 64, 32767])
+def test_weighted_mean_extremes_exact(w_max, reduce, flags):
+    """Eq. 1 / Eq. 2 on voxels of every weight up to the cap, values at both ends of the code range and at the
+    roundings' ties, and on scans that put thousands of contributions into one voxel."""
+    p = synth.params_dict((32, 32, 32), 0.1, 0.3, w_max, 0.2, 0.1, 6.0, reduce, (-16, -16, -16), flags)
+    rng = np.random.default_rng(w_max + reduce)
+    value = rng.choice(np.array([-32767, -32766, -1, 0, 1, 2, 16383, 32766, 32767], np.int16), (32, 32, 32))
+    weight = rng.integers(0, w_max + 1, (32, 32, 32)).astype(np.int16)
+    weight[::2] = w_max
+    pose = synth.pose12(np.eye(3), np.zeros(3))
+    pts = _points(3000, 3, 0.3, 1.5)
+    pts[::3] = np.array([0.9, 0.4, 0.1, 0.0], np.float32)
+    steps = [("scan", pts, pose)] * 2
+    assert_same(run_gpu(p, steps, torch, prefill=(value, weight)), run_oracle(p, steps, prefill=(value, weight)), "mean")
