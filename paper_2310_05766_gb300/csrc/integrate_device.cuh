@@ -817,9 +817,11 @@ __device__ __forceinline__ void apply_staged(const MapDev& m, int32_t w_max, int
 }
 
 // Eq. 1 / Eq. 2 of one voxel without branches, for the usual case of
-// decode_apply: a 32-bit sum, a count below 2^15, a non-negative weight; any
-// other sets bits of `wide` (the caller then takes decode_apply). An untouched
-// voxel keeps its word.
+// decode_apply: a 32-bit sum, a count below 2^15, a non-negative weight (SCAN,
+// the per-scan weight reading: weight times count below 2^15); any other sets
+// bits of `wide` (the caller then takes decode_apply). An untouched voxel keeps
+// its word. With gm = gw (SCAN: gw W), both readings are
+// (gv gm + S) / (gm + W).
 //
 // The rounded quotient (half away from zero) is estimated as the nearest
 // integer to num times an approximate reciprocal of den, taken 2^-19 too small,
@@ -830,7 +832,7 @@ __device__ __forceinline__ void apply_staged(const MapDev& m, int32_t w_max, int
 // step away from zero, when twice the remainder reaches den, corrects it.
 // (The integer pipe bounds the apply, so the products and the rounding run on
 // the other pipes: 320 -> 180 instructions per task of four voxels a lane.)
-template <int MODE>
+template <int MODE, bool SCAN>
 __device__ __forceinline__ void apply_voxel_fast(unsigned long long P, uint32_t& word, int32_t w_max, unsigned& wide,
                                                  unsigned& touched, unsigned& hits) {
     const unsigned lo = (unsigned)P, hi = (unsigned)(P >> 32);
@@ -850,15 +852,17 @@ __device__ __forceinline__ void apply_voxel_fast(unsigned long long P, uint32_t&
     }
     const int gv = (int)(int16_t)(word & 0xFFFFu);
     const int gw = (int)word >> 16;
-    const int num = gv * gw + S;
-    const int den = gw + (int)W;
+    const int gm = SCAN ? gw * (int)W : gw;
+    if (SCAN) wide |= (unsigned)gm & 0xFFFF8000u;
+    const int num = gv * gm + S;
+    const int den = gm + (int)W;
     float rc;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(__int2float_rn(den)));
     rc = fm(rc, 1.0f - 0x1p-19f);
     int q = __float_as_int(__fmaf_rn(__int2float_rn(num), rc, 12582912.0f)) - 0x4B400000;
     const int rem = num - q * den;
     if (2 * abs(rem) >= den) q += (num >> 31) | 1;
-    const int nw = min(den, w_max);
+    const int nw = min(SCAN ? gw + 1 : den, w_max);
     if (W != 0u) {
         word = __byte_perm((unsigned)q, (unsigned)nw, 0x5410);
         ++touched;
@@ -881,21 +885,28 @@ __device__ __forceinline__ unsigned contributions(unsigned long long P) {
     return MODE == 0 ? (unsigned)((P - (unsigned long long)S) >> 40) : (P != 0ull ? 1u : 0u);
 }
 
+template <int MODE, bool SCAN, int NV>
+__device__ __forceinline__ void apply_pairs_fast(int32_t w_max, const ulonglong2 (&acc)[NV], uint2 (&g)[NV],
+                                                 unsigned& wide, unsigned& cnt, unsigned& h) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        // (a row is an 8 x 8 slice of the brick: 28 % of a listed brick's are untouched)
+        if (!__any_sync(kFull, (acc[v].x | acc[v].y) != 0ull)) continue;
+        apply_voxel_fast<MODE, SCAN>(acc[v].x, g[v].x, w_max, wide, cnt, h);
+        apply_voxel_fast<MODE, SCAN>(acc[v].y, g[v].y, w_max, wide, cnt, h);
+    }
+}
+
 // The voxels of a lane's NV pairs: accumulators acc, grid words g (updated),
 // read from gsrc (where they still are).
 template <int MODE, int NV>
 __device__ __forceinline__ void apply_pairs(int32_t w_max, int32_t flags, const ulonglong2 (&acc)[NV], uint2 (&g)[NV],
                                             const uint2* gsrc, unsigned long long& touched, unsigned long long& hits) {
     const unsigned lane = threadIdx.x & 31u;
-    unsigned cnt = 0, h = 0, wide = MODE == 0 ? (unsigned)(flags & kFlagScanWeight) : 0u;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        // (a row is an 8 x 8 slice of the brick: 28 % of a listed brick's are untouched)
-        if (!__any_sync(kFull, (acc[v].x | acc[v].y) != 0ull)) continue;
-        apply_voxel_fast<MODE>(acc[v].x, g[v].x, w_max, wide, cnt, h);
-        apply_voxel_fast<MODE>(acc[v].y, g[v].y, w_max, wide, cnt, h);
-    }
-    if (wide) {   // some voxel outside the usual case, or the per-scan weight reading: this lane again
+    unsigned cnt = 0, h = 0, wide = 0;
+    if (MODE == 0 && (flags & kFlagScanWeight)) apply_pairs_fast<MODE, MODE == 0, NV>(w_max, acc, g, wide, cnt, h);
+    else apply_pairs_fast<MODE, false, NV>(w_max, acc, g, wide, cnt, h);
+    if (wide) {   // some voxel outside the usual case: this lane again
         cnt = h = 0;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
