@@ -5,6 +5,7 @@
 // beyond the per-map constants 1/voxel, QMAX/tau and K, derived once in
 // binary64 and rounded to binary32.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -153,7 +154,10 @@ struct tsdf_map {
     bool chain_merge = false;
     bool chain_pdl = false;
     long long* host_last = nullptr; // mapped pinned copy of the published counters (host address)
-    double* reg_dev = nullptr;      // registration: the 29 sums of the normal equations
+    double* reg_dev = nullptr;      // registration: the CTAs' sums, the 29 sums of the normal equations, a counter
+    double reg_serial = 0.0;        // registration: evaluations so far
+    double* reg_host = nullptr;     // registration: mapped pinned copy of the 29 sums (host address), or null
+    RegisterBuffers reg{};
     size_t pair_cap_req = 0;        // sort reduction: requested pair capacity, 0 = from the scan size
     size_t pool_req = 0;            // pool reduction: requested slots, 0 = default
     // TSDF_REDUCTION_AUTO: the atomic, sort and pool reductions are timed on
@@ -283,6 +287,7 @@ void free_map(tsdf_map* m) {
     cudaFree(m->dev.ctr);
     if (m->host_last) cudaFreeHost(m->host_last);
     cudaFree(m->reg_dev);
+    if (m->reg_host) cudaFreeHost(m->reg_host);
     cudaFree(m->dev.pool_table);
     cudaFree(m->dev.pool_brick);
     cudaFree(m->dev.pool_acc);
@@ -1581,6 +1586,35 @@ int tsdf_extract_mesh(tsdf_map* map, int32_t min_weight, float* out_dev, int64_t
     return TSDF_OK;
 }
 
+// Registration buffers, on first use: kRegisterMaxCtas x 32 sums, the system
+// (where no mapped host memory could be had) and the arrival counter.
+static int ensure_register(tsdf_map* map) {
+    if (map->reg_dev) return TSDF_OK;
+    constexpr size_t kSums = (size_t)kRegisterMaxCtas * 32;
+    double* d = nullptr;
+    TSDF_CU(cudaMalloc(&d, (kSums + 32 + 1) * sizeof(double)));
+    cudaError_t e = cudaMemset(d, 0, (kSums + 32 + 1) * sizeof(double));
+    if (e != cudaSuccess) {
+        cudaFree(d);
+        return cuda_fail(e);
+    }
+    map->reg.part = d;
+    map->reg.out = d + kSums;
+    map->reg.done = reinterpret_cast<unsigned*>(d + kSums + 32);
+    void* dp = nullptr;
+    if (cudaHostAlloc(&map->reg_host, 32 * sizeof(double), cudaHostAllocMapped) == cudaSuccess &&
+        cudaHostGetDevicePointer(&dp, map->reg_host, 0) == cudaSuccess) {
+        std::memset(map->reg_host, 0, 32 * sizeof(double));
+        map->reg.out = static_cast<double*>(dp);
+    } else {
+        if (map->reg_host) cudaFreeHost(map->reg_host);
+        map->reg_host = nullptr;
+        cudaGetLastError();
+    }
+    map->reg_dev = d;
+    return TSDF_OK;
+}
+
 int tsdf_register_system(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12],
                          int32_t min_weight, double* out_host, void* stream) {
     if (!map || !pose || !out_host || n < 0 || n > TSDF_MAX_POINTS || min_weight < 1 || min_weight > 32767)
@@ -1590,12 +1624,30 @@ int tsdf_register_system(tsdf_map* map, const float* points_dev, int64_t n, cons
         if (!std::isfinite(pose[i])) return TSDF_ERR_INVALID;
     DeviceScope ds(map->device);
     cudaStream_t s = (cudaStream_t)stream;
-    if (!map->reg_dev) TSDF_CU(cudaMalloc(&map->reg_dev, 29 * sizeof(double)));
+    int rc = ensure_register(map);
+    if (rc != TSDF_OK) return rc;
     const long long o[3] = {map->origin[0], map->origin[1], map->origin[2]};
     TSDF_CU(launch_register(points_dev, (int)n, pose, map->dev.grid, map->geom, o, map->p.voxel_size, map->inv_vs,
-                            map->p.tau, min_weight, map->reg_dev, s));
-    TSDF_CU(cudaMemcpyAsync(out_host, map->reg_dev, 29 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    TSDF_CU(cudaStreamSynchronize(s));
+                            map->p.tau, min_weight, map->num_sms, map->reg, ++map->reg_serial, s));
+    if (map->reg_host) {
+        // the kernel's last CTA writes the serial behind the sums: watching it
+        // saves the wake-up of a stream synchronisation (all earlier work on
+        // the stream is then over too). The stream is asked now and then, so a
+        // failed launch ends the wait.
+        const volatile double* mark = map->reg_host + 31;
+        for (unsigned polls = 1; *mark != map->reg_serial; ++polls) {
+            if (polls % 4096u != 0u) continue;
+            const cudaError_t e = cudaStreamQuery(s);
+            if (e == cudaSuccess) break;
+            if (e != cudaErrorNotReady) return cuda_fail(e);
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        if (*mark != map->reg_serial) TSDF_CU(cudaStreamSynchronize(s));
+        std::memcpy(out_host, map->reg_host, 29 * sizeof(double));
+    } else {
+        TSDF_CU(cudaMemcpyAsync(out_host, map->reg.out, 29 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        TSDF_CU(cudaStreamSynchronize(s));
+    }
     return TSDF_OK;
 }
 

@@ -257,9 +257,21 @@ cudaError_t launch_sort_apply(const MapDev& m, int32_t reduce, int32_t w_max, in
 cudaError_t launch_shift(uint32_t* grid, const ShiftItem* items, int count, unsigned* claimed, int* claim,
                          cudaStream_t s);
 cudaError_t launch_copy_chunks(const ChunkCopy* items, int count, cudaStream_t s);
+// Registration: device memory for the CTAs' sums (32 doubles each) and their
+// arrival counter (0 between calls), and the device-visible address of the 29
+// sums of the normal equations (mapped host memory, or device memory): 32
+// doubles, the last of which gets the evaluation's serial number when the sums
+// are complete.
+constexpr int kRegisterCtasPerSm = 1;
+constexpr int kRegisterMaxCtas = 512;
+struct RegisterBuffers {
+    double* part;
+    unsigned* done;
+    double* out;
+};
 cudaError_t launch_register(const float* pts_dev, int n, const float pose[12], const uint32_t* grid,
                             const WindowGeom& geo, const long long origin[3], float vs, float inv_vs, float tau,
-                            int min_w, double* out_dev, cudaStream_t s);
+                            int min_w, int sms, const RegisterBuffers& buf, double serial, cudaStream_t s);
 bool register_step(const double sys[29], float pose[12], double* step_norm);
 cudaError_t launch_mesh(const uint32_t* grid, const WindowGeom& geo, const long long origin[3], int min_w, float vs,
                         float* out, unsigned long long cap, unsigned long long* count, cudaStream_t s);
