@@ -752,12 +752,12 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
     const bool fused = scan_fused(a.n);
     cudaError_t e = cudaSuccess;
     if (fused) {
-        e = launch_scan(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
+        e = launch_scan(a, d, map->p.reduce, map->merge, false, map->kpt, map->pdl, cs);
     } else {
-        e = launch_rays(a, d, false, true, map->pdl, cs);
-        if (e == cudaSuccess) e = launch_contrib(a, d, map->p.reduce, map->merge, map->kpt, map->pdl, cs);
+        e = launch_rays(a, d, false, map->pdl, cs);
+        if (e == cudaSuccess) e = launch_contrib(a, d, map->p.reduce, map->merge, false, map->kpt, map->pdl, cs);
     }
-    if (e == cudaSuccess) e = launch_apply(d, (uint32_t)map->bricks, map->p.reduce, map->p.w_max, map->p.flags, map->pdl, cs);
+    if (e == cudaSuccess) e = launch_apply(d, (uint32_t)map->bricks, false, map->p.reduce, map->p.w_max, map->p.flags, map->pdl, cs);
     cudaGraph_t g = nullptr;
     const cudaError_t ee = cudaStreamEndCapture(cs, &g);
     if (e != cudaSuccess || ee != cudaSuccess || !g) {
@@ -768,7 +768,7 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
     // the kernel nodes whose arguments change from scan to scan: the one kernel
     // of a small scan (kept as the contribution node), or ray set-up and
     // contribution
-    const void* fr = fused ? nullptr : rays_kernel_fn(false, true);
+    const void* fr = fused ? nullptr : rays_kernel_fn(false);
     const void* fc = fused ? scan_kernel_fn(map->p.reduce, map->merge) : contrib_kernel_fn(map->p.reduce, map->merge);
     size_t nn = 0;
     std::vector<cudaGraphNode_t> nodes;
@@ -861,26 +861,8 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
     ScanArgs a;
     fill_scan_args(map, points_dev, n, pose, a);
     const bool pdl = map->pdl;
-    if (reduction == TSDF_REDUCTION_POOL) {
-        rc = ensure_rays(map, n);
-        if (rc == TSDF_OK) rc = ensure_pool(map);
-        if (rc != TSDF_OK) return rc;
-        const MapDev& d = map->dev;
-        cudaEvent_t e0 = n > 0 ? prof_mark(map, s) : nullptr;
-        TSDF_CU(launch_rays(a, d, false, false, pdl, s));
-        cudaEvent_t e1 = n > 0 ? prof_mark(map, s) : nullptr;
-        cudaEvent_t e2 = n > 0 ? prof_mark(map, s) : nullptr;
-        TSDF_CU(launch_pool_contrib(a, d, map->p.reduce, map->kpt, pdl, s));
-        cudaEvent_t e3 = n > 0 ? prof_mark(map, s) : nullptr;
-        cudaEvent_t e4 = prof_mark(map, s);
-        TSDF_CU(launch_pool_apply(d, map->p.reduce, map->p.w_max, map->p.flags, pdl, s));   // + counters
-        cudaEvent_t e5 = prof_mark(map, s);
-        prof_push(map, kRays, e0, e1);
-        prof_push(map, kContrib, e2, e3);
-        prof_push(map, kApply, e4, e5);
-        return TSDF_OK;
-    }
-    rc = ensure_acc(map);
+    const bool pool = reduction == TSDF_REDUCTION_POOL;
+    rc = pool ? ensure_pool(map) : ensure_acc(map);
     if (rc != TSDF_OK) return rc;
     if (reduction == TSDF_REDUCTION_SORT) {
         rc = ensure_rays(map, n);
@@ -888,7 +870,7 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
         if (rc != TSDF_OK) return rc;
         const MapDev& d = map->dev;
         cudaEvent_t e0 = n > 0 ? prof_mark(map, s) : nullptr;
-        TSDF_CU(launch_rays(a, d, true, false, pdl, s));
+        TSDF_CU(launch_rays(a, d, true, pdl, s));
         cudaEvent_t e1 = n > 0 ? prof_mark(map, s) : nullptr;
         cudaEvent_t e2 = n > 0 ? prof_mark(map, s) : nullptr;
         TSDF_CU(launch_emit(a, d, map->p.reduce, map->kpt, pdl, s));
@@ -913,7 +895,7 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
         rc = ensure_rays(map, n);
         if (rc != TSDF_OK) return rc;
     }
-    if (n > 0 && map->use_graph && !map->graph_broken && !map->prof) {
+    if (n > 0 && !pool && map->use_graph && !map->graph_broken && !map->prof) {
         bool launched = false;
         rc = chain_graph_launch(map, a, s, &launched);
         if (launched || rc != TSDF_OK) return rc;
@@ -922,15 +904,15 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!fused) {
         e0 = prof_mark(map, s);
-        TSDF_CU(launch_rays(a, map->dev, false, true, pdl, s));
+        TSDF_CU(launch_rays(a, map->dev, false, pdl, s));
         e1 = prof_mark(map, s);
     }
     cudaEvent_t e2 = n > 0 ? prof_mark(map, s) : nullptr;
-    TSDF_CU(fused ? launch_scan(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s)
-                  : launch_contrib(a, map->dev, map->p.reduce, map->merge, map->kpt, pdl, s));
+    TSDF_CU(fused ? launch_scan(a, map->dev, map->p.reduce, map->merge, pool, map->kpt, pdl, s)
+                  : launch_contrib(a, map->dev, map->p.reduce, map->merge, pool, map->kpt, pdl, s));
     cudaEvent_t e3 = n > 0 ? prof_mark(map, s) : nullptr;
     cudaEvent_t e4 = prof_mark(map, s);
-    TSDF_CU(launch_apply(map->dev, (uint32_t)map->bricks, map->p.reduce, map->p.w_max, map->p.flags, pdl, s));
+    TSDF_CU(launch_apply(map->dev, (uint32_t)map->bricks, pool, map->p.reduce, map->p.w_max, map->p.flags, pdl, s));
     cudaEvent_t e5 = prof_mark(map, s);
     prof_push(map, kRays, e0, e1);
     prof_push(map, kContrib, e2, e3);

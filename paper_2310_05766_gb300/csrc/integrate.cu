@@ -116,14 +116,28 @@ using namespace dev;
 #endif
 constexpr int kRaysThreads = TSDF_RAYS_THREADS;
 
-template <bool SORT, bool SPLIT>
+template <bool SORT>
 __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, const MapDev m) {
     __shared__ RaysSmemT<kRaysThreads / 32> sm;
     if constexpr (SORT)
         rays_task_sort<true, kRaysThreads / 32>(a, m, (int)(blockIdx.x * blockDim.x), blockIdx.x, &sm);
     else
-        rays_task_ppt<true, SPLIT, kRaysThreads / 32, kRaysPPT>(a, m, (int)(blockIdx.x * blockDim.x) * kRaysPPT,
+        rays_task_ppt<true, true, kRaysThreads / 32, kRaysPPT>(a, m, (int)(blockIdx.x * blockDim.x) * kRaysPPT,
                                                                 blockIdx.x, &sm);
+}
+
+template <bool POOL>
+__device__ __forceinline__ void cache_init(uint32_t* btab) {
+    for (int i = threadIdx.x; i < (POOL ? 2 * kSlotCache : kBrickCache); i += blockDim.x) btab[i] = kNoVoxel;
+}
+
+// The CTA's cache for a march: of marked bricks, or (pool reduction) of claimed
+// slots; `btab` filled with ones is empty as either.
+template <bool POOL>
+__device__ __forceinline__ BrickCache march_cache(uint32_t* btab) {
+    BrickCache bc{btab, 32u - kBrickCacheLog2};
+    bc.slots = POOL ? reinterpret_cast<unsigned long long*>(btab) : nullptr;
+    return bc;
 }
 
 // Contribution work items: (block of 32 consecutive live rays, group of KPT
@@ -138,18 +152,18 @@ __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, co
 // extra time in brick-flag stores.
 constexpr int kContribThreads = 256;
 
-template <int MODE, bool MERGE>
+template <int MODE, bool MERGE, bool POOL>
 __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contrib_kernel(const ScanArgs a,
                                                                                         const MapDev m,
-                                                                                        const int kpt) {
+                                                                                        const int kpt_max) {
     __shared__ unsigned long long red[kContribThreads / 32];
-    __shared__ uint32_t btab[kBrickCache];
+    __shared__ __align__(8) uint32_t btab[POOL ? 2 * kSlotCache : kBrickCache];   // POOL: the slot cache
     const unsigned lane = threadIdx.x & 31u;
     const unsigned gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    __shared__ unsigned s_counts[2];
+    __shared__ unsigned s_counts[3];
     pdl_trigger();
-    brick_cache_init(btab);
+    cache_init<POOL>(btab);
     pdl_wait();   // ray list and live count come from the rays kernel
     // A coherent load after the wait (a read-only __ldg could be hoisted above
     // it and see a count from before the rays kernel finished), one per CTA:
@@ -161,11 +175,22 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     if (threadIdx.x == 0) {
         s_counts[0] = __ldcg(&m.ctr->live[m.parity].front);
         s_counts[1] = __ldcg(&m.ctr->live[m.parity].back);
+        s_counts[2] = __ldcg(&m.ctr->live[m.parity].fill);
     }
     __syncthreads();   // (also orders the brick cache initialisation)
     const unsigned nf = s_counts[0], nb = s_counts[1];
     const unsigned bf = (nf + 31u) / 32u, bb = (nb + 31u) / 32u;
-    const unsigned ngrp = (unsigned)(2 * a.K + kpt) / (unsigned)kpt;   // ceil((2K+1) / kpt)
+    const unsigned steps = (unsigned)(2 * a.K + 1);
+    // Steps per item: an item of long steps (high fill columns) is cut while the
+    // items are too few to even out over the warps. A 33 k-point corridor scan
+    // of 18 lines (some hundred samples a step): 52 -> 28 us; corridor 64x1024
+    // 24.6 -> 23.2, outdoor 64x1024 19.1 -> 18.4. Items of short steps stay
+    // whole (one of 256^3 voxels at 0.1 m, no fill: 10.5 us with four steps, 12.3
+    // with one), as do those of larger scans (corridor 128x2048: 29.2 and 33.3).
+    const float per_step = 1.f + 2.f * (float)s_counts[2] / (float)max(nf + nb, 1u);   // samples of a mean ray
+    int kpt = kpt_max;
+    while (kpt > 1 && (float)kpt * per_step > 14.f && (bf + bb) * ((steps + kpt - 1) / kpt) < 2u * nwarps) kpt >>= 1;
+    const unsigned ngrp = (steps + kpt - 1) / kpt;
     const unsigned nitems = (bf + bb) * ngrp;
     // first ray of block `blk` and the end of its part of the list
     auto block_ray = [&](unsigned blk, unsigned& end) {
@@ -178,7 +203,8 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     };
     unsigned hits = 0;
     unsigned last_brick = kNoVoxel;
-    const BrickCache bc{btab, 32u - kBrickCacheLog2};
+    uint32_t last_slot = kPoolEmpty;
+    const BrickCache bc = march_cache<POOL>(btab);
     float4 A, B;
     {
         unsigned end;
@@ -191,8 +217,8 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
         unsigned end;
         const unsigned r0 = block_ray(next / ngrp, end);
         load_rays(m, next < nitems ? end : 0u, r0 + lane, An, Bn);   // prefetch
-        contrib_item<MODE, MERGE>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
-                                                      nullptr, bc);
+        contrib_item<MODE, MERGE, false, POOL>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
+                                               &last_slot, bc);
         A = An;
         B = Bn;
     }
@@ -219,12 +245,12 @@ constexpr int kScanThreads = kScanWarps * 32;
 // 5760-point scan: 180 CTAs of one 32-ray block, nine steps over eight warps;
 // through the ray list 14.3 us of contributions, here 12.0 with the set-up,
 // and 17.9 instead of 26.2 us for the whole scan).
-template <int MODE, bool MERGE>
+template <int MODE, bool MERGE, bool POOL>
 __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(const ScanArgs a, const MapDev m,
                                                                                const int tile, const int parts,
                                                                                const int kpt_max) {
     __shared__ float4 s_a[kScanThreads], s_b[kScanThreads];
-    __shared__ uint32_t btab[kBrickCache];
+    __shared__ __align__(8) uint32_t btab[POOL ? 2 * kSlotCache : kBrickCache];   // POOL: the slot cache
     __shared__ unsigned s_heavy[kScanWarps], s_light[kScanWarps], s_valid[kScanWarps];
     __shared__ unsigned s_next;
     __shared__ unsigned long long red[kScanWarps];
@@ -238,7 +264,7 @@ __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
     if (in) p = __ldg(a.pts + i);   // the caller's points: no dependency on earlier grids
     pdl_trigger();
-    brick_cache_init(btab);
+    cache_init<POOL>(btab);
     if (threadIdx.x == 0) s_next = kScanWarps;
     unsigned nlive, nheavy;
     {
@@ -291,7 +317,8 @@ __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(
     const unsigned nitems = blocks * ngrp;
     unsigned hits = 0;
     unsigned last_brick = kNoVoxel;
-    const BrickCache bc{btab, 32u - kBrickCacheLog2};
+    uint32_t last_slot = kPoolEmpty;
+    const BrickCache bc = march_cache<POOL>(btab);
     unsigned claim = warp;
     for (;;) {
         const unsigned item = claim * (unsigned)parts + part;
@@ -302,8 +329,8 @@ __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(
             A = s_a[ray];
             B = s_b[ray];
         }
-        contrib_item<MODE, MERGE>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
-                                                      nullptr, bc);
+        contrib_item<MODE, MERGE, false, POOL>(a, m, item % ngrp, kpt, A, B, hits, last_brick, kNoSlot, nullptr,
+                                               &last_slot, bc);
         if (lane == 0) claim = atomicAdd(&s_next, 1u);
         claim = __shfl_sync(kFull, claim, 0);
     }
@@ -349,36 +376,6 @@ __global__ void __launch_bounds__(256, TSDF_EMIT_MIN_CTAS) emit_kernel(const Sca
     }
 }
 
-// Pool reduction: the contribution march accumulating into claimed pool
-// bricks (same work items as contrib_kernel).
-template <int MODE, int KPT>
-__global__ void __launch_bounds__(256) pool_contrib_kernel(const ScanArgs a, const MapDev m) {
-    __shared__ unsigned long long red[8];
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    pdl_trigger();
-    pdl_wait();
-    unsigned nlive = 0;
-    if (lane == 0) nlive = __ldcg(&m.ctr->live_count);
-    nlive = __shfl_sync(kFull, nlive, 0);
-    const unsigned ngrp = (unsigned)(2 * a.K + KPT) / KPT;
-    const unsigned nitems = (nlive + 31u) / 32u * ngrp;
-    unsigned hits = 0;
-    unsigned last_brick = kNoVoxel;
-    uint32_t last_slot = kPoolEmpty;
-    for (unsigned item = gwarp; item < nitems; item += nwarps) {   // warp-uniform
-        float4 A, B;
-        load_rays(m, nlive, (item / ngrp) * 32u + lane, A, B);
-        contrib_item<MODE, false, false, true>(a, m, item % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
-                                                    &last_slot);
-    }
-    if (MODE == 1) {
-        const unsigned long long total = cta_sum<8>((unsigned long long)hits, red);
-        if (threadIdx.x == 0 && total) atomicAdd(&m.ctr->part[blockIdx.x % kParts].hits, total);
-    }
-}
-
 __global__ void __launch_bounds__(256) sort_count_kernel(const MapDev m) {
     pdl_trigger();
     pdl_wait();   // pairs come from emit, brick slots from compact
@@ -417,13 +414,15 @@ constexpr int kApplyWarps = 4;   // CTA size of the sort and pool apply kernels
 
 // ---- apply of the plain path: one CTA per SM.
 //
-// FLAGS (windows of at most kFlagBricks bricks): every CTA reads ALL brick
+// Flags (windows of at most kFlagBricks bricks): every CTA reads ALL brick
 // flags (64 KB for 512x512x128 voxels, from L2), ranks the touched bricks with
 // one CTA-wide prefix sum and takes every gridDim-th of them, so there is no
 // compaction kernel, no list in memory and no list read before each task. The
 // flags are cleared when all CTAs have read them: the last one to say so has
 // one warp do it while the others work on. Larger windows: the compaction
-// kernel lists the bricks, and each CTA takes every gridDim-th entry.
+// kernel lists the bricks, and each CTA takes every gridDim-th entry. Pool
+// reduction: the claimed slots are the list; their table entries are reset,
+// and when the pool was full the scan is dropped (accumulators cleared only).
 //
 // The CTA's bricks are cut into quarter-brick warp tasks. What bounds them is
 // the latency of their loads (1.5 KB a task), so each warp keeps kApplyStages
@@ -540,7 +539,9 @@ __device__ __forceinline__ unsigned list_own_bricks(const uint8_t* flag, uint32_
     return total;
 }
 
-template <int MODE, bool FLAGS>
+enum ApplySource { kFromFlags, kFromList, kFromPool };
+
+template <int MODE, int SRC>
 __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m, const uint32_t bricks,
                                                                 const unsigned ginv, const int32_t w_max,
                                                                 const int32_t flags) {
@@ -553,12 +554,20 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m,
     pdl_wait();      // flags or list, and accumulators, come from the earlier kernels
     pdl_trigger();   // (after the wait: the next scan's ray set-up writes the ray list)
     unsigned nb;
-    if (FLAGS) {
+    bool dropped = false;   // pool: some brick found it full, the scan only clears up after itself
+    if (SRC == kFromFlags) {
         nb = list_own_bricks(m.brick_flag, bricks, c, G, ginv, s_list, s_warp);
     } else {
-        if (threadIdx.x == 0) s_warp[0] = __ldcg(&m.ctr->brick_count);
+        if (threadIdx.x == 0) {
+            s_warp[0] = __ldcg(SRC == kFromList ? &m.ctr->brick_count : &m.ctr->pool_count);
+            s_warp[1] = SRC == kFromPool ? __ldcg(&m.ctr->pool_overflow) : 0u;
+        }
         __syncthreads();
         nb = s_warp[0];
+        if (SRC == kFromPool) {
+            nb = min(nb, m.pool_cap);
+            dropped = s_warp[1] != 0u;
+        }
     }
     long long* pub = m.host_last ? m.host_last : m.ctr->pub;
     if (warp == kApplyWarpsPlain - 1) {
@@ -569,8 +578,8 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m,
             __threadfence();
         }
         if (__shfl_sync(kFull, last, 0)) {   // all CTAs have read the flags (the list's length): clear them
-            if (!FLAGS) {
-                if (lane == 0) m.ctr->brick_count = 0u;
+            if (SRC != kFromFlags) {
+                if (lane == 0) m.ctr->brick_count = m.ctr->pool_count = m.ctr->pool_overflow = 0u;
             } else if (bricks < 16u) {
                 if (lane < bricks) m.brick_flag[lane] = 0;
             } else {
@@ -591,11 +600,11 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m,
         }
         if (lane == 0) {
             pub[0] = (long long)__ldcg(&lc->valid);
-            pub[1] = (long long)h;
+            pub[1] = dropped ? 0 : (long long)h;
             pub[2] = 0;
-            pub[3] = 0;
+            pub[3] = dropped ? kStatusCapacity : 0;
             pub[4] = (long long)G;
-            lc->front = lc->back = lc->valid = 0u;
+            lc->front = lc->back = lc->valid = lc->fill = 0u;
         }
     }
     // ---- warp tasks: quarters of the CTA's bricks, kApplyStages in flight
@@ -604,19 +613,29 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m,
     unsigned long long touched = 0, hits = 0;
     for (unsigned b0 = 0; b0 < mine; b0 += kApplyList) {   // CTA-uniform; one round unless a list is very long
         const unsigned nl = min(mine - b0, (unsigned)kApplyList);
-        if (!FLAGS) {
+        if (SRC != kFromFlags) {
             __syncthreads();
-            for (unsigned i = threadIdx.x; i < nl; i += kApplyThreads)
-                s_list[i] = __ldcg(m.brick_list + c + (size_t)(b0 + i) * G);
+            for (unsigned i = threadIdx.x; i < nl; i += kApplyThreads) {
+                const size_t at = c + (size_t)(b0 + i) * G;
+                const uint32_t brick = __ldcg((SRC == kFromList ? m.brick_list : m.pool_brick) + at);
+                s_list[i] = brick;
+                if (SRC == kFromPool) m.pool_table[brick] = kPoolEmpty;
+            }
             __syncthreads();
         }
+        // accumulators of task t: the brick's own, or its pool slot's
+        auto acc_word = [&](unsigned t, size_t v) {
+            if (SRC != kFromPool) return v;
+            return ((size_t)(c + (size_t)(b0 + t / kApplyParts) * G) << 9) + (t % kApplyParts) * 128u;
+        };
+        unsigned long long* const accs = SRC == kFromPool ? m.pool_acc : m.acc;
         const unsigned ntask = nl * kApplyParts;
         auto fetch = [&](unsigned t, unsigned stage) {
             if (t < ntask) {
                 const size_t v = ((size_t)s_list[t / kApplyParts] << 9) + (t % kApplyParts) * 128u;
                 ulonglong2* sa = reinterpret_cast<ulonglong2*>(ring + stage * kStageBytes);
                 uint2* sg = reinterpret_cast<uint2*>(ring + stage * kStageBytes + 1024);
-                const ulonglong2* ga = reinterpret_cast<const ulonglong2*>(m.acc + v);
+                const ulonglong2* ga = reinterpret_cast<const ulonglong2*>(accs + acc_word(t, v));
                 const uint2* gg = reinterpret_cast<const uint2*>(m.grid + v);
                 cp_async16(sa + lane, ga + lane);
                 cp_async16(sa + 32 + lane, ga + 32 + lane);
@@ -635,9 +654,10 @@ __global__ void __launch_bounds__(kApplyThreads, 1) apply_kernel(const MapDev m,
             const uint2* sg = reinterpret_cast<const uint2*>(ring + stage * kStageBytes + 1024);
             ulonglong2 acc[kApplyPairs] = {sa[lane], sa[32 + lane]};
             uint2 g[kApplyPairs] = {sg[lane], sg[32 + lane]};
-            apply_pairs<MODE, kApplyPairs>(w_max, flags, acc, g, sg, touched, hits);
+            if (!dropped) apply_pairs<MODE, kApplyPairs>(w_max, flags, acc, g, sg, touched, hits);   // (else the grid words as they were)
             fetch(t + kApplyStages * kApplyWarpsPlain, stage);
-            store_pairs<kApplyPairs>(reinterpret_cast<uint2*>(m.grid + v), reinterpret_cast<ulonglong2*>(m.acc + v), acc, g);
+            store_pairs<kApplyPairs>(reinterpret_cast<uint2*>(m.grid + v),
+                                     reinterpret_cast<ulonglong2*>(accs + acc_word(t, v)), acc, g);
             stage = stage + 1u == kApplyStages ? 0u : stage + 1u;
         }
         cp_async_wait<0>();
@@ -710,63 +730,6 @@ __global__ void __launch_bounds__(kApplyWarps * 32) sort_apply_kernel(const MapD
     finish_if_last(m, &s_last);
 }
 
-
-// Pool reduction: one warp per claimed slot applies Eq. 1 / Eq. 2 to its
-// brick (unless the pool overflowed: then the scan is dropped and the slots
-// are only cleared), resets the slot and the brick's table entry; the last CTA
-// publishes the counters and the scan's status.
-template <int MODE>
-__global__ void __launch_bounds__(kApplyWarps * 32) pool_apply_kernel(const MapDev m, const int32_t w_max,
-                                                                       const int32_t flags) {
-    __shared__ unsigned long long red_u[kApplyWarps], red_h[kApplyWarps];
-    __shared__ unsigned s_last;
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned w = threadIdx.x >> 5;
-    const unsigned gwarp = blockIdx.x * kApplyWarps + w;
-    const unsigned nwarps = gridDim.x * kApplyWarps;
-    pdl_wait();
-    pdl_trigger();   // (after the wait: the next scan's ray set-up writes the ray list)
-    unsigned ns = 0, ovf = 0;
-    if (lane == 0) {
-        ns = __ldcg(&m.ctr->pool_count);
-        ovf = __ldcg(&m.ctr->pool_overflow);
-    }
-    ns = __shfl_sync(kFull, ns, 0);
-    ovf = __shfl_sync(kFull, ovf, 0);
-    if (ns > m.pool_cap) ns = m.pool_cap;
-    unsigned long long touched = 0, hits = 0;
-    for (unsigned i = gwarp; i < ns; i += nwarps) {
-        const unsigned brick = __ldcg(m.pool_brick + i);
-        unsigned long long* accp = m.pool_acc + ((size_t)i << 9);
-        if (!ovf) {
-            apply_brick_at<MODE>(m, w_max, flags, brick, accp, touched, hits);
-        } else {
-            ulonglong2* ap = reinterpret_cast<ulonglong2*>(accp);
-#pragma unroll
-            for (int v = 0; v < 8; ++v) ap[32 * v + lane] = make_ulonglong2(0ull, 0ull);
-        }
-        if (lane == 0) m.pool_table[brick] = kPoolEmpty;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        touched += __shfl_xor_sync(kFull, touched, o);
-        hits += __shfl_xor_sync(kFull, hits, o);
-    }
-    if (lane == 0) {
-        red_u[w] = touched;
-        red_h[w] = hits;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long bu = 0, bh = 0;
-        for (int k = 0; k < kApplyWarps; ++k) {
-            bu += red_u[k];
-            bh += red_h[k];
-        }
-        if (bu) atomicAdd(&m.ctr->part[blockIdx.x % kParts].touched, bu);
-        if (MODE == 0 && bh) atomicAdd(&m.ctr->part[blockIdx.x % kParts].hits, bh);
-    }
-    finish_if_last(m, &s_last);
-}
 
 // Launch with `smem` bytes of dynamic shared memory, with programmatic stream
 // serialisation when `pdl` is set.
@@ -872,35 +835,30 @@ ScanShape scan_shape(int64_t n, int K) {
     return g;
 }
 
+// The kernel of the given mode, merge and pool reduction among a template's instances.
+#define TSDF_PICK(kernel, reduce, merge, pool)                                         \
+    ((pool) ? ((reduce) == 0 ? kernel<0, false, true> : kernel<1, false, true>)        \
+            : (merge) ? ((reduce) == 0 ? kernel<0, true, false> : kernel<1, true, false>) \
+                      : ((reduce) == 0 ? kernel<0, false, false> : kernel<1, false, false>))
+
 const void* scan_kernel_fn(int32_t reduce, bool merge) {
-    if (reduce == 0)
-        return merge ? reinterpret_cast<const void*>(scan_kernel<0, true>)
-                     : reinterpret_cast<const void*>(scan_kernel<0, false>);
-    return merge ? reinterpret_cast<const void*>(scan_kernel<1, true>)
-                 : reinterpret_cast<const void*>(scan_kernel<1, false>);
+    return reinterpret_cast<const void*>(TSDF_PICK(scan_kernel, reduce, merge, false));
 }
 
-cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
+cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, bool pool, int kpt, bool pdl,
                         cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
     const ScanShape g = scan_shape(a.n, a.K);
-    auto* k = reduce == 0 ? (merge ? scan_kernel<0, true> : scan_kernel<0, false>)
-                          : (merge ? scan_kernel<1, true> : scan_kernel<1, false>);
-    return launch(k, dim3(g.grid), dim3(kScanThreads), s, pdl, a, m, g.tile, g.parts, kpt);
+    return launch(TSDF_PICK(scan_kernel, reduce, merge, pool), dim3(g.grid), dim3(kScanThreads), s, pdl, a, m, g.tile,
+                  g.parts, kpt);
 }
 
-const void* rays_kernel_fn(bool sort, bool split) {
-    if (sort) return reinterpret_cast<const void*>(rays_kernel<true, false>);
-    return split ? reinterpret_cast<const void*>(rays_kernel<false, true>)
-                 : reinterpret_cast<const void*>(rays_kernel<false, false>);
+const void* rays_kernel_fn(bool sort) {
+    return sort ? reinterpret_cast<const void*>(rays_kernel<true>) : reinterpret_cast<const void*>(rays_kernel<false>);
 }
 
 const void* contrib_kernel_fn(int32_t reduce, bool merge) {
-    if (reduce == 0)
-        return merge ? reinterpret_cast<const void*>(contrib_kernel<0, true>)
-                     : reinterpret_cast<const void*>(contrib_kernel<0, false>);
-    return merge ? reinterpret_cast<const void*>(contrib_kernel<1, true>)
-                 : reinterpret_cast<const void*>(contrib_kernel<1, false>);
+    return reinterpret_cast<const void*>(TSDF_PICK(contrib_kernel, reduce, merge, false));
 }
 
 unsigned rays_grid(int64_t n, bool sort) {
@@ -908,19 +866,16 @@ unsigned rays_grid(int64_t n, bool sort) {
     return (unsigned)((n + per_cta - 1) / per_cta);
 }
 
-cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool split, bool pdl, cudaStream_t s) {
+cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool pdl, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
-    const dim3 grid(rays_grid(a.n, sort)), block(kRaysThreads);
-    if (sort) return launch(rays_kernel<true, false>, grid, block, s, pdl, a, m);
-    return split ? launch(rays_kernel<false, true>, grid, block, s, pdl, a, m)
-                 : launch(rays_kernel<false, false>, grid, block, s, pdl, a, m);
+    return launch(sort ? rays_kernel<true> : rays_kernel<false>, dim3(rays_grid(a.n, sort)), dim3(kRaysThreads), s,
+                  pdl, a, m);
 }
 
-cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
-                           cudaStream_t s) {
+cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, bool pool, int kpt,
+                           bool pdl, cudaStream_t s) {
     if (a.n <= 0) return cudaSuccess;
-    auto* k = reduce == 0 ? (merge ? contrib_kernel<0, true> : contrib_kernel<0, false>)
-                          : (merge ? contrib_kernel<1, true> : contrib_kernel<1, false>);
+    auto* k = TSDF_PICK(contrib_kernel, reduce, merge, pool);
     return launch(k, resident_grid(k, kContribThreads, TSDF_CONTRIB_CTAS_PER_SM), dim3(kContribThreads), s, pdl, a, m,
                   kpt);
 }
@@ -939,30 +894,6 @@ cudaError_t launch_emit(const ScanArgs& a, const MapDev& m, int32_t reduce, int 
         case 4: return launch_emit_k<1, 4>(a, m, pdl, s);
         default: return launch_emit_k<1, 1>(a, m, pdl, s);
     }
-}
-
-cudaError_t launch_pool_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, int kpt, bool pdl,
-                                cudaStream_t s) {
-    if (a.n <= 0) return cudaSuccess;
-    auto pick = [&](auto* k) { return launch(k, resident_grid(k, 256, TSDF_CONTRIB_CTAS_PER_SM), dim3(256), s, pdl, a, m); };
-    if (reduce == 0) {
-        switch (kpt) {
-            case 2: return pick(pool_contrib_kernel<0, 2>);
-            case 4: return pick(pool_contrib_kernel<0, 4>);
-            default: return pick(pool_contrib_kernel<0, 1>);
-        }
-    }
-    switch (kpt) {
-        case 2: return pick(pool_contrib_kernel<1, 2>);
-        case 4: return pick(pool_contrib_kernel<1, 4>);
-        default: return pick(pool_contrib_kernel<1, 1>);
-    }
-}
-
-cudaError_t launch_pool_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
-                              cudaStream_t s) {
-    auto* k = reduce == 0 ? pool_apply_kernel<0> : pool_apply_kernel<1>;
-    return launch(k, resident_grid(k, kApplyWarps * 32), dim3(kApplyWarps * 32), s, pdl, m, w_max, flags);
 }
 
 cudaError_t launch_sort_count(const MapDev& m, bool pdl, cudaStream_t s) {
@@ -989,17 +920,18 @@ cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStrea
     return launch(compact_kernel, dim3((nwords + 255u) / 256u), dim3(256), s, pdl, m, nwords);
 }
 
-cudaError_t launch_apply(const MapDev& m, uint32_t bricks, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
-                         cudaStream_t s) {
-    const unsigned sms = resident_grid(apply_kernel<0, true>, kApplyThreads, 1).x;
+cudaError_t launch_apply(const MapDev& m, uint32_t bricks, bool pool, int32_t reduce, int32_t w_max, int32_t flags,
+                         bool pdl, cudaStream_t s) {
+    const unsigned sms = resident_grid(apply_kernel<0, kFromFlags>, kApplyThreads, 1).x;
     const unsigned G = std::min(sms, (unsigned)kMaxApplyCtas);
-    const bool by_flags = bricks <= kFlagBricks && (bricks + G - 1) / G <= (uint32_t)kApplyList;
-    if (!by_flags) {
+    const bool by_flags = !pool && bricks <= kFlagBricks && (bricks + G - 1) / G <= (uint32_t)kApplyList;
+    if (!pool && !by_flags) {
         const cudaError_t e = launch_compact(m, bricks, pdl, s);
         if (e != cudaSuccess) return e;
     }
-    auto* k = by_flags ? (reduce == 0 ? apply_kernel<0, true> : apply_kernel<1, true>)
-                       : (reduce == 0 ? apply_kernel<0, false> : apply_kernel<1, false>);
+    auto* k = pool ? (reduce == 0 ? apply_kernel<0, kFromPool> : apply_kernel<1, kFromPool>)
+              : by_flags ? (reduce == 0 ? apply_kernel<0, kFromFlags> : apply_kernel<1, kFromFlags>)
+                         : (reduce == 0 ? apply_kernel<0, kFromList> : apply_kernel<1, kFromList>);
     const cudaError_t e = allow_smem(reinterpret_cast<const void*>(k), kApplySmem);
     if (e != cudaSuccess) return e;
     const unsigned ginv = (unsigned)(((1ull << 32) + G - 1) / G);

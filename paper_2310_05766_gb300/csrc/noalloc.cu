@@ -183,14 +183,14 @@ extern "C" int tsdf_integrate_static(uint32_t* grid_dev, const tsdf_params* para
     bool launched_contrib = false;
     if (e == cudaSuccess) {
         if (scan_fused(n)) {
-            e = launch_scan(a, md, params->reduce, false, 4, true, s);
+            e = launch_scan(a, md, params->reduce, false, false, 4, true, s);
         } else {
-            e = launch_rays(a, md, false, true, true, s);
-            if (e == cudaSuccess) e = launch_contrib(a, md, params->reduce, false, 4, true, s);
+            e = launch_rays(a, md, false, true, s);
+            if (e == cudaSuccess) e = launch_contrib(a, md, params->reduce, false, false, 4, true, s);
         }
         launched_contrib = true;
     }
-    if (e == cudaSuccess) e = launch_apply(md, (uint32_t)bricks, params->reduce, params->w_max, params->flags, true, s);
+    if (e == cudaSuccess) e = launch_apply(md, (uint32_t)bricks, false, params->reduce, params->w_max, params->flags, true, s);
     if (e == cudaSuccess && stats_host) {
         long long pub[kPubWords] = {}, last[3] = {0, 0, 0};
         e = cudaMemcpyAsync(pub, md.ctr->pub, sizeof(pub), cudaMemcpyDeviceToHost, s);

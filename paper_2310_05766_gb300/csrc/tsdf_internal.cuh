@@ -38,11 +38,12 @@ constexpr int kMaxApplyCtas = 160;
 constexpr int kPubWords = 8 + 2 * kMaxApplyCtas;
 
 // Rays of a plain scan (split ray list): heavy ones from the list's front,
-// light ones from its end, and valid points. Two of them, used in turn by
+// light ones from its end, valid points, and the sum of the rays' fill heights
+// (voxels each side at the hit, 255 at most). Two of them, used in turn by
 // consecutive scans (MapDev::parity): the ray set-up counts into one while the
 // previous scan's apply still reads and clears the other.
 struct LiveCounts {
-    unsigned int front, back, valid, pad;
+    unsigned int front, back, valid, fill;
 };
 
 struct MapCounters {
@@ -207,10 +208,11 @@ int map_reserve_points(::tsdf_map* map, int64_t n);
 int map_reserve_sort(::tsdf_map* map, int64_t n);
 
 // Launchers (return the cudaError_t of the launch).
-// sort: reserve pair slots per ray (sort reduction); split: heavy rays (fill
-// of at least one voxel each side) from the list's front, the others from
-// its end (the contribution kernel takes heavy work first).
-cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool split, bool pdl, cudaStream_t s);
+// Ray set-up into the map's ray list. sort: pair slots per ray too (sort
+// reduction); otherwise heavy rays (fill of at least one voxel each side) from
+// the list's front, the others from its end (the contribution kernel takes
+// heavy work first).
+cudaError_t launch_rays(const ScanArgs& a, const MapDev& m, bool sort, bool pdl, cudaStream_t s);
 // Plain atomic path up to the list of touched bricks: one kernel over tiles
 // of points for small scans, else ray set-up and the contribution kernel
 // (scan_fused tells which; the ray list is needed only by the latter).
@@ -226,26 +228,21 @@ unsigned rays_grid(int64_t n, bool sort);
 // The kernel functions that these launchers launch for these arguments (to
 // find their nodes in a captured graph).
 const void* scan_kernel_fn(int32_t reduce, bool merge);
-const void* rays_kernel_fn(bool sort, bool split);
+const void* rays_kernel_fn(bool sort);
 const void* contrib_kernel_fn(int32_t reduce, bool merge);
-cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
+// (pool: contributions into claimed pool slots)
+cudaError_t launch_scan(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, bool pool, int kpt, bool pdl,
                         cudaStream_t s);
-cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, int kpt, bool pdl,
-                           cudaStream_t s);
+cudaError_t launch_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, bool merge, bool pool, int kpt,
+                           bool pdl, cudaStream_t s);
 cudaError_t launch_compact(const MapDev& m, uint32_t bricks, bool pdl, cudaStream_t s);
-// Eq. 1 / Eq. 2 on the bricks whose flags are set (and the flags' reset, and
-// the scan's counters).
-cudaError_t launch_apply(const MapDev& m, uint32_t bricks, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
-                         cudaStream_t s);
+// Eq. 1 / Eq. 2 on the bricks whose flags are set, or (pool) that have slots;
+// the flags' or slots' reset, and the scan's counters.
+cudaError_t launch_apply(const MapDev& m, uint32_t bricks, bool pool, int32_t reduce, int32_t w_max, int32_t flags,
+                         bool pdl, cudaStream_t s);
 // Sort reduction: emit pairs, count per brick, prefix, scatter, reduce + apply.
 cudaError_t launch_emit(const ScanArgs& a, const MapDev& m, int32_t reduce, int kpt, bool pdl, cudaStream_t s);
 cudaError_t launch_sort_count(const MapDev& m, bool pdl, cudaStream_t s);
-// Pool reduction: the contribution march into claimed pool bricks, and the
-// apply over the claimed slots (which also publishes the counters).
-cudaError_t launch_pool_contrib(const ScanArgs& a, const MapDev& m, int32_t reduce, int kpt, bool pdl,
-                                cudaStream_t s);
-cudaError_t launch_pool_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
-                              cudaStream_t s);
 cudaError_t launch_sort_scan(const MapDev& m, bool pdl, cudaStream_t s);
 cudaError_t launch_sort_scatter(const MapDev& m, bool pdl, cudaStream_t s);
 cudaError_t launch_sort_apply(const MapDev& m, int32_t reduce, int32_t w_max, int32_t flags, bool pdl,
