@@ -446,8 +446,6 @@ __device__ __forceinline__ uint32_t cached_pool_slot(const MapDev& m, unsigned b
 //    at least 2^22 as an unsigned number. So `rel < dims` (unsigned) is
 //    exactly the window test o <= f < o + dims, and (rel + o mod dims) mod
 //    dims the ring index, for any finite f;
-//  * x and y in packed binary32 pairs (each lane of a pair is an IEEE
-//    round-to-nearest operation, as the scalar ones);
 //  * fill samples +j and -j share the offset B * (j vs): the oracle's
 //    b + B * (-(j vs)) is exactly b - B * (j vs), and the j = 0 sample is b
 //    itself (b + B * 0 rounds to b, up to the sign of a zero, which changes
@@ -456,67 +454,56 @@ __device__ __forceinline__ uint32_t cached_pool_slot(const MapDev& m, unsigned b
 //    rounding never leaves [-32767, 32767].
 constexpr uint32_t kMagicBits = 0x4B400000u;   // bit pattern of 1.5 * 2^23
 
-__device__ __forceinline__ float2 f2(float x, float y) { return make_float2(x, y); }
+// What a sample of the lean march reads of its scan and map, as values: the
+// batched kernel keeps both in shared memory, where every store to the brick
+// cache would have them read again sample by sample; a march copies them into
+// registers once. (The per-map kernels have them in constant memory: nothing
+// changes for those.)
+struct LeanConst {
+    float inv_vs, vs, mx, my, mz, ntx, nty, ntz, tau, qs;
+    uint32_t omb[3], dmask[3], cy, cz;
+    unsigned long long* acc;
+    __device__ __forceinline__ LeanConst(const ScanArgs& a, const MapDev& m)
+        : inv_vs(a.inv_vs), vs(a.vs), mx(a.l_m.x), my(a.l_m.y), mz(a.l_mz), ntx(a.l_nt.x), nty(a.l_nt.y),
+          ntz(a.l_ntz), tau(a.tau), qs(a.qs), omb{a.l_omb[0], a.l_omb[1], a.l_omb[2]},
+          dmask{a.dmask[0], a.dmask[1], a.dmask[2]}, cy(a.l_cy), cz(a.l_cz), acc(m.acc) {}
+};
 
-// Packed (x, y) binary32 add and multiply, each component round-to-nearest.
-// TSDF_LEAN_PACKED selects where packed pairs are used: bit 0 for the sample
-// position (b, q, q / vs, the window add), bit 1 for the voxel centre and the
-// projection; 0 = scalar operations throughout.
-#ifndef TSDF_LEAN_PACKED
-#define TSDF_LEAN_PACKED 0
-#endif
-template <bool PACKED>
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    if (PACKED) return __fadd2_rn(a, b);
-    return make_float2(fa(a.x, b.x), fa(a.y, b.y));
-}
-template <bool PACKED>
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-    if (PACKED) return __fmul2_rn(a, b);
-    return make_float2(fm(a.x, b.x), fm(a.y, b.y));
-}
-constexpr bool kPackPos = (TSDF_LEAN_PACKED & 1) != 0;
-constexpr bool kPackCtr = (TSDF_LEAN_PACKED & 2) != 0;
-
-// One sample at q = (qxy, qz) of a ray (direction A, range r): voxel, code,
-// reduction and brick mark. `mine` = the lane's ray has this sample.
+// One sample at q of a ray (direction A, range r): voxel, code, reduction and
+// brick mark. `mine` = the lane's ray has this sample.
 // last_brick / last_slot: what the lane visited last on this side of the ray
 // (+j and -j samples alternate, each side moving on by one voxel, so each keeps
 // its own).
 template <int MODE, bool SV, bool POOL>
-__device__ __forceinline__ void lean_sample(const ScanArgs& a, const MapDev& m, float2 qxy,
-                                            float qz, const float4& A, float dstep, bool mine, unsigned& hits,
+__device__ __forceinline__ void lean_sample(const LeanConst& c, const MapDev& m, float qx, float qy, float qz,
+                                            const float4& A, float dstep, bool mine, unsigned& hits,
                                             unsigned& last_brick, uint32_t& last_slot, const BrickCache& bc) {
-    const float2 yxy = mul2<kPackPos>(qxy, a.l_inv);
-    const float yz = fm(qz, a.inv_vs);
-    const float fx = floorf(yxy.x), fy = floorf(yxy.y), fz = floorf(yz);
-    const float2 uxy = add2<kPackPos>(f2(fx, fy), a.l_m);
-    const float uz = fa(fz, a.l_mz);
-    const uint32_t bx = __float_as_uint(uxy.x), by = __float_as_uint(uxy.y), bz = __float_as_uint(uz);
-    const bool act = mine && (bx - kMagicBits < a.l_dim[0]) && (by - kMagicBits < a.l_dim[1]) &&
-                     (bz - kMagicBits < a.l_dim[2]);
+    const float fx = floorf(fm(qx, c.inv_vs)), fy = floorf(fm(qy, c.inv_vs)), fz = floorf(fm(qz, c.inv_vs));
+    const uint32_t bx = __float_as_uint(fa(fx, c.mx)), by = __float_as_uint(fa(fy, c.my)),
+                   bz = __float_as_uint(fa(fz, c.mz));
+    const bool act = mine && (bx - kMagicBits <= c.dmask[0]) && (by - kMagicBits <= c.dmask[1]) &&
+                     (bz - kMagicBits <= c.dmask[2]);
     // ring coordinates and the bricked word index:
     // word = sx + 8 sy + 64 sz + 504 (sx >> 3) + cy (sy >> 3) + cz (sz >> 3)
-    const uint32_t sx = (bx + a.l_omb[0]) & a.dmask[0];
-    const uint32_t sy = (by + a.l_omb[1]) & a.dmask[1];
-    const uint32_t sz = (bz + a.l_omb[2]) & a.dmask[2];
-    const uint32_t word = sx + (sy << 3) + (sz << 6) + (sx >> 3) * 504u + (sy >> 3) * a.l_cy + (sz >> 3) * a.l_cz;
+    const uint32_t sx = (bx + c.omb[0]) & c.dmask[0];
+    const uint32_t sy = (by + c.omb[1]) & c.dmask[1];
+    const uint32_t sz = (bz + c.omb[2]) & c.dmask[2];
+    const uint32_t word = sx + (sy << 3) + (sz << 6) + (sx >> 3) * 504u + (sy >> 3) * c.cy + (sz >> 3) * c.cz;
     float d;
     if (SV) {
         d = dstep;
     } else {
         // projective distance of the voxel centre (f + 0.5) vs
-        const float2 cxy = mul2<kPackCtr>(add2<kPackCtr>(f2(fx, fy), f2(0.5f, 0.5f)), a.l_vs);
-        const float cz = fm(fa(fz, 0.5f), a.vs);
-        const float2 exy = mul2<kPackCtr>(add2<kPackCtr>(cxy, a.l_nt), f2(A.x, A.y));
-        const float ez = fm(fa(cz, a.l_ntz), A.z);
-        d = fs(A.w, fa(fa(exy.x, exy.y), ez));
+        const float ex = fm(fa(fm(fa(fx, 0.5f), c.vs), c.ntx), A.x);
+        const float ey = fm(fa(fm(fa(fy, 0.5f), c.vs), c.nty), A.y);
+        const float ez = fm(fa(fm(fa(fz, 0.5f), c.vs), c.ntz), A.z);
+        d = fs(A.w, fa(fa(ex, ey), ez));
     }
-    d = fminf(fmaxf(d, -a.tau), a.tau);
-    const int q = small_int(fm(d, a.qs));
+    d = fminf(fmaxf(d, -c.tau), c.tau);
+    const int q = small_int(fm(d, c.qs));
     if (act) {
         const unsigned brick = word >> 9;
-        unsigned long long* dst = m.acc + word;
+        unsigned long long* dst = c.acc + word;
         if (POOL) {
             // the accumulators of the brick's slot; no brick flags: the claimed
             // slots list the touched bricks
@@ -547,31 +534,31 @@ template <int MODE, bool SV, bool POOL>
 __device__ __forceinline__ void lean_march(const ScanArgs& a, const MapDev& m, int k0, int kpt, const float4& A,
                                            const float4& B, unsigned& hits, unsigned& last_brick,
                                            uint32_t& last_slot, const BrickCache& bc) {
+    const LeanConst c(a, m);
     const float r = A.w;                // dead lanes carry r = -1
     const bool rfill = B.w != 0.f;
     unsigned low_brick = kNoVoxel;      // the -j side's last brick and slot
     uint32_t low_slot = kPoolEmpty;
+    const int K = a.K;
 #pragma unroll 1
     for (int kk = 0; kk < kpt; ++kk) {
         const int k = k0 + kk;
-        if (k > a.K) break;   // uniform
+        if (k > K) break;   // uniform
         float l;
         const int J = step_fill(a, r, rfill, k, l);   // -1: no sample
         const int Jw = __reduce_max_sync(kFull, J);
         if (Jw < 0) continue;   // uniform
-        const float2 bxy = add2<kPackPos>(a.l_t, mul2<kPackPos>(f2(A.x, A.y), f2(l, l)));
-        const float bz = fa(a.t[2], fm(A.z, l));
+        const float bx = fa(a.t[0], fm(A.x, l)), by = fa(a.t[1], fm(A.y, l)), bz = fa(a.t[2], fm(A.z, l));
         const float dstep = fs(r, l);
-        lean_sample<MODE, SV, POOL>(a, m, bxy, bz, A, dstep, J >= 0, hits, last_brick, last_slot, bc);
+        lean_sample<MODE, SV, POOL>(c, m, bx, by, bz, A, dstep, J >= 0, hits, last_brick, last_slot, bc);
         for (int j = 1; j <= Jw; ++j) {   // warp-uniform bounds
-            const float jd = fm((float)j, a.vs);
-            const float2 oxy = mul2<kPackPos>(f2(B.x, B.y), f2(jd, jd));
-            const float oz = fm(B.z, jd);
+            const float jd = fm((float)j, c.vs);
+            const float ox = fm(B.x, jd), oy = fm(B.y, jd), oz = fm(B.z, jd);
             const bool mine = j <= J;
-            lean_sample<MODE, SV, POOL>(a, m, add2<kPackPos>(bxy, oxy), fa(bz, oz), A, dstep, mine, hits, last_brick,
+            lean_sample<MODE, SV, POOL>(c, m, fa(bx, ox), fa(by, oy), fa(bz, oz), A, dstep, mine, hits, last_brick,
                                         last_slot, bc);
-            lean_sample<MODE, SV, POOL>(a, m, add2<kPackPos>(bxy, f2(-oxy.x, -oxy.y)), fs(bz, oz), A, dstep, mine, hits,
-                                        low_brick, low_slot, bc);
+            lean_sample<MODE, SV, POOL>(c, m, fs(bx, ox), fs(by, oy), fs(bz, oz), A, dstep, mine, hits, low_brick,
+                                        low_slot, bc);
         }
     }
 }
