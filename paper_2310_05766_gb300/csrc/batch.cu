@@ -459,7 +459,7 @@ struct tsdf_batch {
         unsigned char* dev = nullptr;
         cudaEvent_t done = nullptr;        // recorded after the set's launch
         bool pending = false;
-        cudaGraphExec_t exec[kNumConfigs] = {};
+        cudaGraphExec_t exec[2][kNumConfigs] = {};   // by grid (its share of the device, or all of it)
     } slot[2];
     int next_slot = 0;
     BatchSync* sync = nullptr;
@@ -503,8 +503,9 @@ struct DevScope {
 void free_batch(tsdf_batch* b) {
     if (!b) return;
     for (auto& s : b->slot) {
-        for (auto& e : s.exec)
-            if (e) cudaGraphExecDestroy(e);
+        for (auto& g : s.exec)
+            for (auto& e : g)
+                if (e) cudaGraphExecDestroy(e);
         if (s.host) cudaFreeHost(s.host);
         cudaFree(s.dev);
         if (s.done) cudaEventDestroy(s.done);
@@ -519,20 +520,21 @@ void free_batch(tsdf_batch* b) {
 }
 
 // CTAs launched for configuration `cfg`: its co-resident CTAs (limited to
-// ctas_per_sm per SM when set), scaled by the grid-fraction option.
-int grid_of(const tsdf_batch* b, int cfg) {
-    return std::max(1, (int)((long long)b->grid_max[cfg] * b->grid_pct / 100));
+// ctas_per_sm per SM when set), scaled by the grid-fraction option unless the
+// launch takes the whole device.
+int grid_of(const tsdf_batch* b, int cfg, bool whole = false) {
+    return std::max(1, (int)((long long)b->grid_max[cfg] * (whole ? 100 : b->grid_pct) / 100));
 }
 
 // Enqueue copy + barrier reset + cooperative kernel for descriptor slot `si`.
-cudaError_t enqueue(tsdf_batch* b, int si, int cfg, cudaStream_t s) {
+cudaError_t enqueue(tsdf_batch* b, int si, int cfg, bool whole, cudaStream_t s) {
     tsdf_batch::Slot& sl = b->slot[si];
     cudaError_t e = cudaMemcpyAsync(sl.dev, sl.host, b->desc_bytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->sync, 0, sizeof(BatchSync), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     const Config& c = kConfigs[cfg];
-    lc.gridDim = dim3((unsigned)grid_of(b, cfg));
+    lc.gridDim = dim3((unsigned)grid_of(b, cfg, whole));
     lc.blockDim = dim3((unsigned)c.threads);
     lc.dynamicSmemBytes = dyn_smem(c);
     lc.stream = s;
@@ -657,7 +659,7 @@ int tsdf_batch_set_option(tsdf_batch* b, int32_t option, int64_t value) {
                             cudaEventSynchronize(sl.done);
                             sl.pending = false;
                         }
-                        for (auto& e : sl.exec)
+                        for (auto& e : sl.exec[0])   // (the whole-device graphs stay as they are)
                             if (e) {
                                 cudaGraphExecDestroy(e);
                                 e = nullptr;
@@ -700,6 +702,15 @@ int tsdf_batch_get_config(const tsdf_batch* b, int32_t* config, int32_t* merge, 
 
 int tsdf_batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* const* points_dev, const int64_t* n,
                          const float* poses, int32_t count, void* stream) {
+    return batch_integrate(b, maps, points_dev, n, poses, count, false, stream);
+}
+
+}  // extern "C"
+
+namespace tsdf {
+
+int batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* const* points_dev, const int64_t* n,
+                    const float* poses, int32_t count, bool whole, void* stream) {
     if (!b || !maps || !points_dev || !n || !poses || count < 0 || count > b->max_count) return TSDF_ERR_INVALID;
     if (count == 0) return TSDF_OK;
     for (int i = 0; i < count; ++i) {
@@ -768,21 +779,21 @@ int tsdf_batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* cons
     }
     if (e == cudaSuccess) {
         if (b->use_graph) {
-            if (!sl.exec[cfg]) {
+            if (!sl.exec[whole][cfg]) {
                 // capture copy + reset + kernel once for this slot and config
                 cudaGraph_t g = nullptr;
                 e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal);
                 if (e == cudaSuccess) {
-                    cudaError_t e2 = enqueue(b, si, cfg, b->capture_stream);
+                    cudaError_t e2 = enqueue(b, si, cfg, whole, b->capture_stream);
                     e = cudaStreamEndCapture(b->capture_stream, &g);
                     if (e == cudaSuccess) e = e2;
                 }
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec[cfg], g, 0);
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec[whole][cfg], g, 0);
                 if (g) cudaGraphDestroy(g);
             }
-            if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec[cfg], s);
+            if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec[whole][cfg], s);
         } else {
-            e = enqueue(b, si, cfg, s);
+            e = enqueue(b, si, cfg, whole, s);
         }
     }
     if (e == cudaSuccess && timing) {
@@ -798,6 +809,10 @@ int tsdf_batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* cons
     b->next_slot ^= 1;
     return TSDF_OK;
 }
+
+}  // namespace tsdf
+
+extern "C" {
 
 int tsdf_integrate_batch(tsdf_map* const* maps, const float* const* points_dev, const int64_t* n, const float* poses,
                          int32_t count, void* stream) {

@@ -4,7 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
-struct tsdf_map;   // host-side map object (defined in api.cu)
+struct tsdf_map;     // host-side map object (defined in api.cu)
+struct tsdf_batch;   // batch object (defined in batch.cu)
 
 namespace tsdf {
 
@@ -195,6 +196,11 @@ int map_reserve_points(::tsdf_map* map, int64_t n);
 // Grow the map's ray and sort-reduction buffers for scans of n points
 // (synchronous allocation on first use or growth).
 int map_reserve_sort(::tsdf_map* map, int64_t n);
+
+// tsdf_batch_integrate; whole: on all of the device whatever the batch's grid
+// fraction.
+int batch_integrate(::tsdf_batch* batch, ::tsdf_map* const* maps, const float* const* points_dev, const int64_t* n,
+                    const float* poses, int32_t count, bool whole, void* stream);
 
 // Launchers (return the cudaError_t of the launch).
 // Ray set-up into the map's ray list. sort: pair slots per ray too (sort
