@@ -35,11 +35,6 @@
 #include "integrate_device.cuh"
 #include "../../include/tsdf.h"
 
-// 1: the atomic configurations apply each brick from registers
-// (apply_brick_reg); 0: through shared memory (apply_brick).
-#ifndef TSDF_BATCH_APPLY_REG
-#define TSDF_BATCH_APPLY_REG 1
-#endif
 // Voxel pairs per lane in one register-apply task of the atomic configurations
 // (8: a warp per brick, 4: per half brick, 2: per quarter brick). Whole bricks
 // measured fastest here (quarter bricks: 1.85 against 1.67 ms for 64 maps;
@@ -330,8 +325,13 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
     }
 
     // ---- phase 4: Eq. 1 / Eq. 2 on the touched bricks, one warp task per brick
-    // (register apply: per part of a brick, kTaskParts parts each)
-    constexpr unsigned kTaskParts = (!SORT && TSDF_BATCH_APPLY_REG) ? 8u / APAIRS : 1u;
+    // (register apply: per part of a brick, kTaskParts parts each). The tasks go
+    // from the last map to the first: the accumulators of a large batch do not
+    // fit the L2 (32 maps of 512 x 512 x 128: 0.4 GB touched), and those marched
+    // last are still there; the next batch's march then begins with the maps
+    // applied last. Batch of 8 / 16 / 32 / 48 uneven maps: 196 -> 191, 333 ->
+    // 326, 659 -> 654, 862 -> 856 us.
+    constexpr unsigned kTaskParts = SORT ? 1u : 8u / APAIRS;
     block_prefix(count, [&](int i) { return __ldcg(&items[i].m.ctr->brick_count) * kTaskParts; }, s_prefix);
     {
         uint32_t* s_grid = reinterpret_cast<uint32_t*>(dyn + w * kApplySmemPerWarp);
@@ -340,7 +340,8 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
         int cur = -1;
         unsigned long long touched = 0, hits = 0;
         for (uint32_t g = gwarp; g < s_prefix[count]; g += nwarps) {   // warp-uniform
-            const int i = find_segment(s_prefix, count, g);
+            const uint32_t t = s_prefix[count] - 1u - g;
+            const int i = find_segment(s_prefix, count, t);
             if (i != cur) {
                 if (cur >= 0) {
                     warp_add(touched, &items[cur].m.ctr->part[gwarp % kParts].touched);
@@ -356,21 +357,16 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
             }
             const BatchItem& it = items[i];
             const MapDev& im = s_dev[w];
-            const unsigned local = g - s_prefix[i];
+            const unsigned local = t - s_prefix[i];
             if (SORT) {
                 const bool ovf = __ldcg(&im.ctr->overflow) != 0u;
                 if (it.reduce == 0)
                     sort_apply_brick<0>(im, it.w_max, it.flags, local, ovf, s_grid, s_acc, s_off, touched, hits);
                 else sort_apply_brick<1>(im, it.w_max, it.flags, local, ovf, s_grid, s_acc, s_off, touched, hits);
             } else {
-#if TSDF_BATCH_APPLY_REG
                 if (it.reduce == 0)
                     apply_part_reg<0, APAIRS>(im, it.w_max, it.flags, local, touched, hits);
                 else apply_part_reg<1, APAIRS>(im, it.w_max, it.flags, local, touched, hits);
-#else
-                if (it.reduce == 0) apply_brick<0>(im, it.w_max, it.flags, local, s_grid, s_acc, s_off, touched, hits);
-                else apply_brick<1>(im, it.w_max, it.flags, local, s_grid, s_acc, s_off, touched, hits);
-#endif
             }
         }
         if (cur >= 0) {
@@ -421,7 +417,7 @@ constexpr int kNumConfigs = 13;
 // (64-map batch, configuration 0: 1.40 against 1.66 ms).
 size_t dyn_smem(const Config& c) {
     const size_t warps = (size_t)(c.threads / 32);
-    if (c.sort || !TSDF_BATCH_APPLY_REG) return warps * kApplySmemPerWarp;
+    if (c.sort) return warps * kApplySmemPerWarp;
     return std::max<size_t>(4u << kCtaBrickCacheLog2, warps * kWarpCacheBytes);
 }
 

@@ -984,39 +984,6 @@ __device__ __forceinline__ void apply_part_reg(const MapDev& m, int32_t w_max, i
     apply_brick_at<MODE, NV>(m, w_max, flags, brick, m.acc + ((size_t)brick << 9), touched, hits, (t % P) * NV);
 }
 
-// ---- apply: one warp updates listed brick number i of the map. Shared
-// memory per warp: s_grid[512] words, s_acc[512] accumulators, s_off[512].
-template <int MODE>
-__device__ __forceinline__ void apply_brick(const MapDev& m, int32_t w_max, int32_t flags, unsigned i,
-                                            uint32_t* s_grid, unsigned long long* s_acc, uint16_t* s_off,
-                                            unsigned long long& touched, unsigned long long& hits) {
-    const unsigned lane = threadIdx.x & 31u;
-    uint4* sg4 = reinterpret_cast<uint4*>(s_grid);
-    ulonglong2* sa2 = reinterpret_cast<ulonglong2*>(s_acc);
-    const unsigned brick = m.brick_list[i];
-    // coalesced, bank-conflict-free 16-byte copies of the brick into shared
-    // memory: accumulator pair p = 32 v + lane holds voxels 2p and 2p + 1
-    const uint4* gp = reinterpret_cast<const uint4*>(m.grid + ((size_t)brick << 9));
-    ulonglong2* ap = reinterpret_cast<ulonglong2*>(m.acc + ((size_t)brick << 9));
-    unsigned nz = 0;   // bit 2v (2v+1): voxel 2(32 v + lane) (+1) has a non-zero accumulator
-#pragma unroll
-    for (int v = 0; v < 4; ++v) sg4[32 * v + lane] = gp[32 * v + lane];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-        const ulonglong2 a2 = ap[32 * v + lane];
-        sa2[32 * v + lane] = a2;
-        nz |= (a2.x != 0ull ? 1u : 0u) << (2 * v);
-        nz |= (a2.y != 0ull ? 1u : 0u) << (2 * v + 1);
-    }
-    apply_staged<MODE>(m, w_max, flags, brick, nz, s_grid, s_acc, s_off, touched, hits);
-    if (nz) {
-#pragma unroll
-        for (int v = 0; v < 8; ++v)
-            if (nz & (3u << (2 * v))) ap[32 * v + lane] = make_ulonglong2(0ull, 0ull);
-    }
-    __syncwarp();
-}
-
 // ---- sort reduction (counting sort of the emitted pairs by touched brick,
 // then a per-brick segmented reduction in shared memory)
 
