@@ -61,6 +61,12 @@ constexpr uint32_t kTagShift = 22;
 static_assert((4u << kCtaBrickCacheLog2) <= 4 * kApplySmemPerWarp, "CTA brick cache fits four warps' staging");
 static_assert((4u << kCtaBrickCacheLog2) <= 4 * kWarpCacheBytes, "CTA brick cache fits four warps' caches");
 
+// Contribution items per warp from which chunks are claimed (phase 2).
+#ifndef TSDF_BATCH_CLAIM_ITEMS
+#define TSDF_BATCH_CLAIM_ITEMS 32
+#endif
+constexpr unsigned kClaimItems = TSDF_BATCH_CLAIM_ITEMS;
+
 struct BatchHeader {
     int32_t count;
     uint32_t ray_tasks;                      // total CTA ray tasks (THREADS times the configuration's points per thread)
@@ -76,7 +82,7 @@ struct BatchSync {
     unsigned arrive;
     unsigned generation;
     unsigned error;
-    unsigned pad;
+    unsigned next;   // phase 2: chunks of items claimed
 };
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
@@ -179,6 +185,7 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
     __shared__ ScanArgs s_args[kBatchWarps];
     __shared__ MapDev s_dev[kBatchWarps];
     __shared__ RaysSmemT<kBatchWarps> rsm;
+    __shared__ uint32_t s_claim[2];
     const int count = hdr->count;
     const unsigned arrivals = gridDim.x + hdr->extra_arrivals;
     const long long spin = hdr->spin_limit;
@@ -240,54 +247,81 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
         BrickCache bc = cta_cache ? BrickCache{ctab, 32u - kCtaBrickCacheLog2, 0u}
                                   : BrickCache{reinterpret_cast<uint32_t*>(dyn + w * kWarpCacheBytes),
                                                32u - kWarpBrickCacheLog2, 0u};
-        for (uint32_t g = gwarp; g < s_prefix[count]; g += nwarps) {   // warp-uniform
-            const int i = find_segment(s_prefix, count, g);
-            if (i != cur) {
-                if (cur >= 0 && items[cur].reduce == 1)
-                    warp_add(hits, &items[cur].m.ctr->part[gwarp % kParts].hits);
-                if (cur >= 0 && ovf) items[cur].m.ctr->overflow = 1u;
-                hits = 0;
-                ovf = false;
-                last_brick = kNoVoxel;
-                cur = i;
-                if (cta_cache) {
-                    bc.tag = (uint32_t)i << kTagShift;
+        // The items are handed out in chunks of consecutive ones to a whole CTA,
+        // whose warps share the brick cache: with a grid stride while they are
+        // few, else claimed from a counter, one chunk ahead. Items differ in
+        // cost (the last group of a block's steps is short, and a stride that
+        // the number of groups divides gives a warp the same group every
+        // time): CTAs were done 20 to 110 us before the last one of a 400 us
+        // march. Long chunks cost the L2 its reuse (chunks of 2 / 3 / 6 items a
+        // warp, 32 maps of 512 x 512 x 128: 645 / 663 / 710 us), claims of
+        // single warps cost more brick flag stores (727). Static against claimed:
+        // 32 maps 661 and 646 us, 48 maps 865 and 831, 64 small scans 908 and
+        // 800, 32 of them 408 and 390; 16 of them, 24 items a warp, 219 and 228.
+        const uint32_t total = s_prefix[count];
+        const bool claimed = total >= kClaimItems * nwarps;
+        const uint32_t chunk_items = kBatchWarps * (claimed ? 2u : 1u);
+        uint32_t chunk = blockIdx.x;
+        for (unsigned k = 0; chunk * chunk_items < total; ++k) {   // CTA-uniform
+            uint32_t next = 0;
+            if (claimed && threadIdx.x == 0) next = gridDim.x + atomicAdd(&sync->next, 1u);
+            const uint32_t end = min(total, (chunk + 1u) * chunk_items);
+            for (uint32_t g = chunk * chunk_items + w; g < end; g += kBatchWarps) {   // warp-uniform
+                const int i = find_segment(s_prefix, count, g);
+                if (i != cur) {
+                    if (cur >= 0 && items[cur].reduce == 1)
+                        warp_add(hits, &items[cur].m.ctr->part[gwarp % kParts].hits);
+                    if (cur >= 0 && ovf) items[cur].m.ctr->overflow = 1u;
+                    hits = 0;
+                    ovf = false;
+                    last_brick = kNoVoxel;
+                    cur = i;
+                    if (cta_cache) {
+                        bc.tag = (uint32_t)i << kTagShift;
+                    } else {
+                        for (int e = (int)lane; e < (1 << kWarpBrickCacheLog2); e += 32) bc.tab[e] = kNoVoxel;
+                    }
+                    __syncwarp();   // the warp is done with the previous map's copies
+                    {
+                        const uint32_t* sa = reinterpret_cast<const uint32_t*>(&items[i].a);
+                        uint32_t* da = reinterpret_cast<uint32_t*>(&s_args[w]);
+                        for (int e = (int)lane; e < (int)(sizeof(ScanArgs) / 4); e += 32) da[e] = sa[e];
+                        const uint32_t* sm_ = reinterpret_cast<const uint32_t*>(&items[i].m);
+                        uint32_t* dm = reinterpret_cast<uint32_t*>(&s_dev[w]);
+                        for (int e = (int)lane; e < (int)(sizeof(MapDev) / 4); e += 32) dm[e] = sm_[e];
+                    }
+                    __syncwarp();
+                }
+                const BatchItem& it = items[i];
+                const ScanArgs& ia = s_args[w];
+                const MapDev& im = s_dev[w];
+                const unsigned ngrp = (unsigned)(2 * ia.K + KPT) / KPT;
+                const unsigned local = g - s_prefix[i];
+                const unsigned nl = s_live[i];
+                const unsigned ray = (local / ngrp) * 32u + lane;
+                float4 A, B;
+                load_rays(im, nl, ray, A, B);
+                if (SORT) {
+                    const uint32_t sslot = ray < nl ? im.ray_slot[ray] : kNoSlot;
+                    if (it.reduce == 0)
+                        contrib_item<0, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
+                                                          nullptr, bc);
+                    else contrib_item<1, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
+                                                           nullptr, bc);
                 } else {
-                    for (int e = (int)lane; e < (1 << kWarpBrickCacheLog2); e += 32) bc.tab[e] = kNoVoxel;
+                    if (it.reduce == 0)
+                        contrib_item<0, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
+                                                    nullptr, bc);
+                    else contrib_item<1, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
+                                                     nullptr, bc);
                 }
-                __syncwarp();   // the warp is done with the previous map's copies
-                {
-                    const uint32_t* sa = reinterpret_cast<const uint32_t*>(&items[i].a);
-                    uint32_t* da = reinterpret_cast<uint32_t*>(&s_args[w]);
-                    for (int e = (int)lane; e < (int)(sizeof(ScanArgs) / 4); e += 32) da[e] = sa[e];
-                    const uint32_t* sm_ = reinterpret_cast<const uint32_t*>(&items[i].m);
-                    uint32_t* dm = reinterpret_cast<uint32_t*>(&s_dev[w]);
-                    for (int e = (int)lane; e < (int)(sizeof(MapDev) / 4); e += 32) dm[e] = sm_[e];
-                }
-                __syncwarp();
             }
-            const BatchItem& it = items[i];
-            const ScanArgs& ia = s_args[w];
-            const MapDev& im = s_dev[w];
-            const unsigned ngrp = (unsigned)(2 * ia.K + KPT) / KPT;
-            const unsigned local = g - s_prefix[i];
-            const unsigned nl = s_live[i];
-            const unsigned ray = (local / ngrp) * 32u + lane;
-            float4 A, B;
-            load_rays(im, nl, ray, A, B);
-            if (SORT) {
-                const uint32_t sslot = ray < nl ? im.ray_slot[ray] : kNoSlot;
-                if (it.reduce == 0)
-                    contrib_item<0, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
-                                                      nullptr, bc);
-                else contrib_item<1, false, true>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, sslot, &ovf,
-                                                       nullptr, bc);
+            if (claimed) {
+                if (threadIdx.x == 0) s_claim[k & 1u] = next;
+                __syncthreads();
+                chunk = s_claim[k & 1u];
             } else {
-                if (it.reduce == 0)
-                    contrib_item<0, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
-                                                nullptr, bc);
-                else contrib_item<1, MERGE>(ia, im, local % ngrp, KPT, A, B, hits, last_brick, kNoSlot, nullptr,
-                                                 nullptr, bc);
+                chunk += gridDim.x;
             }
         }
         if (cur >= 0 && items[cur].reduce == 1) warp_add(hits, &items[cur].m.ctr->part[gwarp % kParts].hits);
