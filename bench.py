@@ -418,10 +418,11 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
                  note="tsdf_integrate_host from pinned memory (read in place by the first kernel over the host "
                       "link unless --zero-copy 0) + tsdf_stats read-back, host wall clock"),
         # library launches: one per profiled entry, plus the compaction that shares
-        # the apply entry (atomic) or compact + count + prefix + scatter sharing
-        # the sort entry (sort); the pool reduction has no compaction
+        # the apply entry (atomic, windows of more than 65536 bricks only) or
+        # compact + count + prefix + scatter sharing the sort entry (sort); the
+        # pool reduction has no compaction
         gpu_launches=int(sum(v[0] for v in prof.values()) +
-                         {"atomic": 1, "sort": 3, "pool": 0}[args.reduction] * K),
+                         {"atomic": int(np.prod(p["dims"]) // 512 > 65536), "sort": 3, "pool": 0}[args.reduction] * K),
         clocks=clk,
         wall_s_timed=t_wall,
         cpu_baseline=cpu,

@@ -106,7 +106,8 @@ typedef struct tsdf_map tsdf_map;   /* opaque; owns all of its device memory */
  * kept all-zero between calls) is allocated by the first integrate call that
  * uses the atomic or sort reduction (the pool reduction keeps a smaller one of
  * its own), and the per-ray buffers (32 bytes per point) by the first
- * integrate call that needs them. Synchronous. On success *out receives the
+ * integrate call that needs them (one of more than 32768 points, a batched one
+ * or one with the sort reduction). Synchronous. On success *out receives the
  * handle, which the caller releases with tsdf_map_destroy. Errors: INVALID,
  * OOM, CUDA. */
 int tsdf_map_create(const tsdf_params* params, tsdf_map** out);
@@ -128,8 +129,8 @@ int tsdf_map_destroy(tsdf_map* map);
  *                transform [R | t]; R's third column is the direction
  *                orthogonal to the scan lines. Copied at call time.
  * The result is bit-identical to a serial evaluation in any launch order.
- * When n exceeds every earlier n of this map, the per-ray buffers grow first
- * (a synchronous reallocation). Errors: INVALID, OOM, CUDA. */
+ * When a call that needs the per-ray buffers has more points than every earlier
+ * one of this map, they grow first (a synchronous reallocation). Errors: INVALID, OOM, CUDA. */
 int tsdf_integrate(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12], void* stream);
 
 /* As tsdf_integrate, but points_host is a HOST pointer (pinned or pageable)
@@ -267,13 +268,13 @@ int tsdf_stats(tsdf_map* map, tsdf_scan_stats* out, void* stream);
 #define TSDF_OPT_STORE_SPILL_AGE 9  /* global store: a chunk stored this many shifts ago moves from device to
                                       host memory at the next shift; 0 (default): only when the device tier is
                                       full */
-#define TSDF_OPT_LAUNCH_GRAPH 10  /* 1: the atomic reduction's four kernels are captured once into a CUDA
+#define TSDF_OPT_LAUNCH_GRAPH 10  /* 1: the atomic reduction's two to four kernels are captured once into a CUDA
                                     graph (again after buffers or options change) and each scan sets the
                                     graph's arguments and launches it once: less host time per scan, for
-                                    callers whose thread is the bottleneck; 0 (default): four launches per
-                                    scan, which let consecutive scans overlap on the device. Scans while
+                                    callers whose thread is the bottleneck; 0 (default): one launch per
+                                    kernel, which lets consecutive scans overlap on the device. Scans while
                                     profiling is enabled or while the caller's stream is being captured use
-                                    four launches. */
+                                    one launch per kernel. */
 
 /* Device memory held by the map (grid, per-scan buffers of the reductions
  * that have been used, ray buffers, global store) in bytes. Host-side.
@@ -303,7 +304,9 @@ int tsdf_grid_device_ptr(const tsdf_map* map, void** out);
 /* Per-kernel device time of this map's launches, measured with CUDA events
  * recorded on the launching stream around each kernel while profiling is on. */
 typedef struct tsdf_kernel_time {
-    char    name[24];     /* "rays", "contrib", "apply" (brick compaction, update, counters) or "shift" */
+    char    name[24];     /* "rays" (none for scans whose rays are set up by the contribution kernel: up to
+                             32768 points), "contrib", "apply" (in windows of more than 2^16 bricks with the
+                             brick compaction; update, counters) or "shift" */
     int64_t launches;     /* kernel launches since profiling was enabled */
     double  total_ms;     /* summed event-to-event device time */
 } tsdf_kernel_time;
@@ -427,7 +430,7 @@ int tsdf_probe_reduction_rate(int32_t pattern, double* per_second, void* stream)
  * cooperative launch: the phases of tsdf_integrate (ray set-up, contributions,
  * brick compaction, Eq. 1 / Eq. 2 update, counters) run over all maps of the
  * batch with a grid-wide barrier between phases, so maps of uneven size share
- * the whole GPU and a batch costs one launch instead of five per map. Each map's
+ * the whole GPU and a batch costs one launch instead of several per map. Each map's
  * result is bit-identical to tsdf_integrate of the same scan. The launch (a
  * descriptor copy, a barrier reset and the kernel) is captured once into a CUDA
  * graph and replayed; the descriptors are the only thing that changes. */

@@ -133,7 +133,7 @@ struct tsdf_map {
     bool pdl = true;                // programmatic dependent launch between the scan's kernels
     int reduction = TSDF_REDUCTION_ATOMIC;   // per-scan reduction: accumulator atomics or sort
     bool zero_copy = true;          // tsdf_integrate_host reads device-mapped pinned points in place
-    // The plain path's four launches as one CUDA graph (TSDF_OPT_LAUNCH_GRAPH):
+    // The plain path's launches as one CUDA graph (TSDF_OPT_LAUNCH_GRAPH):
     // captured on first use, then per scan the ray and contribution nodes get
     // the scan's arguments and the graph is launched once. Off by default: it
     // cuts the host's time per scan from about 9 to 3.5 us, but back-to-back
@@ -731,7 +731,7 @@ static bool same_dev(const MapDev& x, const MapDev& y) {
            x.pool_acc == y.pool_acc && x.pool_cap == y.pool_cap;
 }
 
-// Capture the plain atomic path (rays, contribution, compaction, apply with
+// Capture the plain atomic path (scan or rays + contribution, apply with
 // the map's options) into chain_graph and instantiate it; false when any step
 // fails (nothing is left half built).
 static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {

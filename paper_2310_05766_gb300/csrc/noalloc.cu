@@ -10,8 +10,8 @@
 // in one file-scope __device__ array of fixed size, which every GPU that loads
 // the library keeps until the process exits.
 //
-// The kernels are the library's integration kernels (rays, contrib, compact,
-// and apply, whose last CTA publishes the counters); only the origin of their
+// The kernels are the library's integration kernels (scan or rays + contrib,
+// then apply, whose CTAs publish the counters); only the origin of their
 // scratch memory differs.
 #include <cmath>
 #include <cstddef>
@@ -49,8 +49,8 @@ std::mutex g_mu;
 unsigned char* g_scratch_ptr[kMaxDevices] = {};
 // Per device: a call failed after its contribution kernel may have written
 // accumulators or brick flags, so the next call clears them. (A call that
-// completes leaves both all zero: the compaction clears the flags it lists
-// and the apply resets every accumulator it reads; a freshly loaded module's
+// completes leaves both all zero: the apply clears the flags once all of its
+// CTAs have read them, and resets every accumulator it reads; a freshly loaded module's
 // array is zero.)
 bool g_dirty[kMaxDevices] = {};
 
