@@ -591,6 +591,20 @@ int tsdf_map_destroy(tsdf_map* map) {
     return TSDF_OK;
 }
 
+// Fills a new allocation and waits for it, on a stream of its own: the call
+// that needs it may launch on any stream, and a fill on the default stream
+// would be ordered neither before that launch nor apart from what the caller
+// has queued there.
+static cudaError_t fill_new(void* p, int byte, size_t bytes) {
+    cudaStream_t t = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, byte, bytes, t);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(t);
+    cudaStreamDestroy(t);
+    return e;
+}
+
 // The dense per-scan accumulator (8 B per voxel, all zero between scans) is
 // allocated on the first call that needs it: the atomic and sort reductions,
 // batches and sessions. A map used only with the pool reduction never holds it.
@@ -598,7 +612,7 @@ static int ensure_acc(tsdf_map* map) {
     if (map->dev.acc) return TSDF_OK;
     unsigned long long* a = nullptr;
     TSDF_CU(cudaMalloc(&a, map->voxels * sizeof(unsigned long long)));
-    cudaError_t e = cudaMemset(a, 0, map->voxels * sizeof(unsigned long long));
+    cudaError_t e = fill_new(a, 0, map->voxels * sizeof(unsigned long long));
     if (e != cudaSuccess) {
         cudaFree(a);
         return cuda_fail(e);
@@ -627,10 +641,10 @@ static int ensure_pool(tsdf_map* map) {
     map->dev.pool_acc = nullptr;
     map->dev.pool_cap = 0;
     TSDF_CU(cudaMalloc(&map->dev.pool_table, map->bricks * sizeof(uint32_t)));
-    TSDF_CU(cudaMemset(map->dev.pool_table, 0xFF, map->bricks * sizeof(uint32_t)));
+    TSDF_CU(fill_new(map->dev.pool_table, 0xFF, map->bricks * sizeof(uint32_t)));
     TSDF_CU(cudaMalloc(&map->dev.pool_brick, want * sizeof(uint32_t)));
     TSDF_CU(cudaMalloc(&map->dev.pool_acc, want * kBrickVoxels * sizeof(unsigned long long)));
-    TSDF_CU(cudaMemset(map->dev.pool_acc, 0, want * kBrickVoxels * sizeof(unsigned long long)));
+    TSDF_CU(fill_new(map->dev.pool_acc, 0, want * kBrickVoxels * sizeof(unsigned long long)));
     map->dev.pool_cap = (uint32_t)want;
     return TSDF_OK;
 }
@@ -660,7 +674,7 @@ static int ensure_sort(tsdf_map* map, int64_t n) {
         TSDF_CU(cudaMalloc(&map->dev.brick_slot, map->bricks * sizeof(uint32_t)));
         TSDF_CU(cudaMalloc(&map->dev.seg_count, map->bricks * sizeof(uint32_t)));
         TSDF_CU(cudaMalloc(&map->dev.seg_start, map->bricks * sizeof(uint32_t)));
-        TSDF_CU(cudaMemset(map->dev.seg_count, 0, map->bricks * sizeof(uint32_t)));
+        TSDF_CU(fill_new(map->dev.seg_count, 0, map->bricks * sizeof(uint32_t)));
     }
     if (map->ray_slot_cap < map->ray_cap) {
         cudaFree(map->dev.ray_slot);

@@ -1,0 +1,59 @@
+"""First use of a map on a side stream while the default stream is busy: the buffers that a call allocates
+then are filled before its kernels run, whatever the default stream still has to do."""
+import numpy as np
+import pytest
+
+from paper_2310_05766_gb300 import synth
+from helpers import assert_same, run_oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _busy_default_stream():
+    """Copies that keep the default stream busy for tens of milliseconds."""
+    a = torch.ones(1 << 28, device="cuda")
+    c = torch.empty_like(a)
+    torch.cuda.synchronize()
+    for _ in range(60):
+        c.copy_(a)
+    return a, c
+
+
+def _dirty_free_memory():
+    """Memory that the next allocations may get back is not zero."""
+    x = torch.full((1 << 26,), 7, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    del x
+    torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("reduction", ["ATOMIC", "SORT", "POOL"])
+@pytest.mark.parametrize("n", [2000, 40000])
+def test_first_scan_on_side_stream(n, reduction):
+    from paper_2310_05766_gb300 import binding as b
+    p = synth.params_dict((128, 128, 64), 0.1, 0.3, 64, 0.05, 0.3, 6.0, 0, (-64, -64, -32))
+    rng = np.random.default_rng(n)
+    d = rng.normal(size=(n, 3))
+    pts = np.zeros((n, 4), np.float32)
+    pts[:, :3] = d / np.linalg.norm(d, axis=1, keepdims=True) * rng.uniform(0.5, 5.0, (n, 1))
+    pose = synth.pose12(synth.rot_zyx(0.3, 0.1, -0.1), np.array([0.05, 0.1, -0.02]))
+    _dirty_free_memory()
+    m = b.TsdfMap(p)
+    try:
+        b.tsdf_set_option(m.handle, b.TSDF_OPT_REDUCTION, getattr(b, "TSDF_REDUCTION_" + reduction))
+        dev = torch.from_numpy(pts).cuda()
+        side = torch.cuda.Stream()
+        busy = _busy_default_stream()
+        with torch.cuda.stream(side):
+            m.integrate(dev, pose)
+            m.integrate(dev, pose)
+            stats = m.stats()
+        torch.cuda.synchronize()
+        del busy
+        v, w = m.read()
+        got = (v, w, [stats], m.origin)
+    finally:
+        m.close()
+    ref = run_oracle(p, [("scan", pts, pose)] * 2)
+    assert_same(got, (ref[0], ref[1], ref[2][-1:], ref[3]), reduction)
