@@ -1589,7 +1589,7 @@ static int ensure_register(tsdf_map* map) {
     constexpr size_t kSums = (size_t)kRegisterMaxCtas * 32;
     double* d = nullptr;
     TSDF_CU(cudaMalloc(&d, (kSums + 32 + 1) * sizeof(double)));
-    cudaError_t e = cudaMemset(d, 0, (kSums + 32 + 1) * sizeof(double));
+    cudaError_t e = fill_new(d, 0, (kSums + 32 + 1) * sizeof(double));
     if (e != cudaSuccess) {
         cudaFree(d);
         return cuda_fail(e);
@@ -1639,6 +1639,7 @@ int tsdf_register_system(tsdf_map* map, const float* points_dev, int64_t n, cons
         }
         std::atomic_thread_fence(std::memory_order_acquire);
         if (*mark != map->reg_serial) TSDF_CU(cudaStreamSynchronize(s));
+        if (*mark != map->reg_serial) return cuda_fail(cudaErrorUnknown);   // the sums are not this evaluation's
         std::memcpy(out_host, map->reg_host, 29 * sizeof(double));
     } else {
         TSDF_CU(cudaMemcpyAsync(out_host, map->reg.out, 29 * sizeof(double), cudaMemcpyDeviceToHost, s));

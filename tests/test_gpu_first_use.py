@@ -3,6 +3,7 @@ then are filled before its kernels run, whatever the default stream still has to
 import numpy as np
 import pytest
 
+import oracle
 from paper_2310_05766_gb300 import synth
 from helpers import assert_same, run_oracle
 
@@ -57,3 +58,35 @@ def test_first_scan_on_side_stream(n, reduction):
         m.close()
     ref = run_oracle(p, [("scan", pts, pose)] * 2)
     assert_same(got, (ref[0], ref[1], ref[2][-1:], ref[3]), reduction)
+
+
+@pytest.mark.parametrize("n", [100, 60001])
+def test_first_registration_on_side_stream(n):
+    from paper_2310_05766_gb300 import binding as b
+    p = synth.params_dict((32, 16, 64), 0.1, 0.3, 64, 0.0, 0.1, 10.0, 0, (-16, 8, -32))
+    rng = np.random.default_rng(n)
+    shape = (64, 16, 32)
+    value = np.rint(np.clip((np.arange(64)[:, None, None] + rng.uniform(-0.4, 0.4, shape) - 20) * 6000, -32767, 32767))
+    value, weight = value.astype(np.int16), rng.integers(1, 5, shape).astype(np.int16)
+    pts = np.zeros((n, 4), np.float32)
+    pts[:, :3] = rng.uniform((-1.5, 0.9, -1.5), (1.5, 2.3, -0.9), (n, 3))
+    pose = synth.pose12(synth.rot_zyx(0.05, -0.02, 0.03), np.array([0.01, 0.02, -0.03]))
+    om = oracle.OracleMap(p)
+    om.load_window(value, weight)
+    ref = om.register_system(pts, pose)
+    _dirty_free_memory()
+    m = b.TsdfMap(p)
+    try:
+        m.write(value, weight)
+        dev = torch.from_numpy(pts).cuda()
+        side = torch.cuda.Stream()
+        busy = _busy_default_stream()
+        with torch.cuda.stream(side):
+            got = [b.tsdf_register_system(m.handle, dev, pose) for _ in range(3)]
+        torch.cuda.synchronize()
+        del busy
+        for g in got:
+            assert g[28] == ref[28] > 0
+            assert np.allclose(g, ref, rtol=1e-9, atol=1e-12 * np.abs(ref).max())
+    finally:
+        m.close()
