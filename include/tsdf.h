@@ -402,7 +402,8 @@ int tsdf_extract_mesh(tsdf_map* map, int32_t min_weight, float* out_dev, int64_t
  * place after each successful step; solve by Cholesky, stops when the step
  * norm falls below 1e-7). result may be NULL. Returns TSDF_ERR_DEGENERATE
  * (pose_inout keeping the last good pose) when a step finds fewer than 6
- * points or a singular system. Errors: INVALID, DEGENERATE, CUDA. */
+ * points or a singular system. Synchronises `stream`. Errors: INVALID,
+ * DEGENERATE, CUDA. */
 typedef struct tsdf_register_result {
     int64_t used_points;  /* points in the last evaluated system */
     double  rms;          /* sqrt(sum d^2 / points) of the last evaluated system, metres */

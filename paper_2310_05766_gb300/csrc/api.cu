@@ -6,6 +6,7 @@
 // binary64 and rounded to binary32.
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -1582,6 +1583,10 @@ int tsdf_extract_mesh(tsdf_map* map, int32_t min_weight, float* out_dev, int64_t
     return TSDF_OK;
 }
 
+// How long a registration watches for an evaluation's sums before it blocks (an
+// evaluation of 2^17 points takes 30 us).
+constexpr int kRegisterWatchUs = 200;
+
 // Registration buffers, on first use: kRegisterMaxCtas x 32 sums, the system
 // (where no mapped host memory could be had) and the arrival counter.
 static int ensure_register(tsdf_map* map) {
@@ -1611,53 +1616,68 @@ static int ensure_register(tsdf_map* map) {
     return TSDF_OK;
 }
 
-int tsdf_register_system(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12],
-                         int32_t min_weight, double* out_host, void* stream) {
-    if (!map || !pose || !out_host || n < 0 || n > TSDF_MAX_POINTS || min_weight < 1 || min_weight > 32767)
-        return TSDF_ERR_INVALID;
-    if (n > 0 && (!points_dev || ((uintptr_t)points_dev & 15u) != 0)) return TSDF_ERR_INVALID;
+static bool register_args_ok(const tsdf_map* map, const float* points_dev, int64_t n, const float* pose,
+                             int32_t min_weight) {
+    if (!map || !pose || n < 0 || n > TSDF_MAX_POINTS || min_weight < 1 || min_weight > 32767) return false;
+    if (n > 0 && (!points_dev || ((uintptr_t)points_dev & 15u) != 0)) return false;
     for (int i = 0; i < 12; ++i)
-        if (!std::isfinite(pose[i])) return TSDF_ERR_INVALID;
-    DeviceScope ds(map->device);
-    cudaStream_t s = (cudaStream_t)stream;
+        if (!std::isfinite(pose[i])) return false;
+    return true;
+}
+
+// One evaluation of the normal equations. When it returns the sums are complete
+// and all earlier work on the stream is over, but the kernel may still be
+// retiring: its caller synchronises the stream before it returns.
+static int register_evaluate(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12],
+                             int32_t min_weight, double* out_host, cudaStream_t s) {
     int rc = ensure_register(map);
     if (rc != TSDF_OK) return rc;
     const long long o[3] = {map->origin[0], map->origin[1], map->origin[2]};
     TSDF_CU(launch_register(points_dev, (int)n, pose, map->dev.grid, map->geom, o, map->p.voxel_size, map->inv_vs,
                             map->p.tau, min_weight, map->num_sms, map->reg, ++map->reg_serial, s));
-    if (map->reg_host) {
-        // the kernel's last CTA writes the serial behind the sums: watching it
-        // saves the wake-up of a stream synchronisation (all earlier work on
-        // the stream is then over too). The stream is asked now and then, so a
-        // failed launch ends the wait.
-        const volatile double* mark = map->reg_host + 31;
-        for (unsigned polls = 1; *mark != map->reg_serial; ++polls) {
-            if (polls % 4096u != 0u) continue;
-            const cudaError_t e = cudaStreamQuery(s);
-            if (e == cudaSuccess) break;
-            if (e != cudaErrorNotReady) return cuda_fail(e);
-        }
-        std::atomic_thread_fence(std::memory_order_acquire);
-        if (*mark != map->reg_serial) TSDF_CU(cudaStreamSynchronize(s));
-        if (*mark != map->reg_serial) return cuda_fail(cudaErrorUnknown);   // the sums are not this evaluation's
-        std::memcpy(out_host, map->reg_host, 29 * sizeof(double));
-    } else {
+    if (!map->reg_host) {
         TSDF_CU(cudaMemcpyAsync(out_host, map->reg.out, 29 * sizeof(double), cudaMemcpyDeviceToHost, s));
         TSDF_CU(cudaStreamSynchronize(s));
+        return TSDF_OK;
     }
+    // The kernel's last CTA writes the serial behind the sums: watching it for
+    // as long as an evaluation takes saves the wake-up of a stream
+    // synchronisation. What takes longer (earlier work on the stream, a failed
+    // launch) is left to the synchronisation, which waits as the program has
+    // asked its device to.
+    const volatile double* mark = map->reg_host + 31;
+    const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(kRegisterWatchUs);
+    for (unsigned polls = 1; *mark != map->reg_serial; ++polls)
+        if (polls % 64u == 0u && std::chrono::steady_clock::now() > until) break;
+    std::atomic_thread_fence(std::memory_order_acquire);
+    if (*mark != map->reg_serial) TSDF_CU(cudaStreamSynchronize(s));
+    if (*mark != map->reg_serial) return cuda_fail(cudaErrorUnknown);   // the sums are not this evaluation's
+    std::memcpy(out_host, map->reg_host, 29 * sizeof(double));
     return TSDF_OK;
 }
 
-int tsdf_register(tsdf_map* map, const float* points_dev, int64_t n, float pose_inout[12], int32_t iterations,
-                  int32_t min_weight, tsdf_register_result* result, void* stream) {
-    if (!pose_inout || iterations < 1 || iterations > 1000) return TSDF_ERR_INVALID;
+int tsdf_register_system(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12],
+                         int32_t min_weight, double* out_host, void* stream) {
+    if (!out_host || !register_args_ok(map, points_dev, n, pose, min_weight)) return TSDF_ERR_INVALID;
+    DeviceScope ds(map->device);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int rc = register_evaluate(map, points_dev, n, pose, min_weight, out_host, s);
+    if (rc != TSDF_OK) return rc;
+    TSDF_CU(cudaStreamSynchronize(s));
+    return TSDF_OK;
+}
+
+static int register_steps(tsdf_map* map, const float* points_dev, int64_t n, float pose_inout[12], int32_t iterations,
+                          int32_t min_weight, tsdf_register_result* result, cudaStream_t s) {
     float pose[12];
     std::memcpy(pose, pose_inout, sizeof(pose));
     double sys[29];
     tsdf_register_result res{};
     int it = 0;
     for (; it < iterations; ++it) {
-        int rc = tsdf_register_system(map, points_dev, n, pose, min_weight, sys, stream);
+        // (a step can leave the finite range: refused like any such pose)
+        if (!register_args_ok(map, points_dev, n, pose, min_weight)) return TSDF_ERR_INVALID;
+        int rc = register_evaluate(map, points_dev, n, pose, min_weight, sys, s);
         if (rc != TSDF_OK) return rc;
         res.used_points = (int64_t)sys[28];
         res.rms = sys[28] > 0 ? std::sqrt(sys[27] / sys[28]) : 0.0;
@@ -1677,6 +1697,18 @@ int tsdf_register(tsdf_map* map, const float* points_dev, int64_t n, float pose_
     res.iterations = it;
     if (result) *result = res;
     return TSDF_OK;
+}
+
+int tsdf_register(tsdf_map* map, const float* points_dev, int64_t n, float pose_inout[12], int32_t iterations,
+                  int32_t min_weight, tsdf_register_result* result, void* stream) {
+    if (iterations < 1 || iterations > 1000 || !register_args_ok(map, points_dev, n, pose_inout, min_weight))
+        return TSDF_ERR_INVALID;
+    DeviceScope ds(map->device);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int rc = register_steps(map, points_dev, n, pose_inout, iterations, min_weight, result, s);
+    const cudaError_t e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess && (rc == TSDF_OK || rc == TSDF_ERR_DEGENERATE)) return cuda_fail(e);
+    return rc;
 }
 
 int tsdf_extract_surface(tsdf_map* map, int32_t min_weight, float* out_dev, int64_t capacity, int64_t* count,

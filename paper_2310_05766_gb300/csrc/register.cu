@@ -187,12 +187,10 @@ __global__ void __launch_bounds__(kRegWarps * 32) register_kernel(const RegArgs 
         for (int w = 1; w < kRegWarps; ++w) s += red[w][lane];
         if (lane < (unsigned)kSysN)
             out[lane] = s * (lane < 21u ? a.f_h : lane < 27u ? a.f_g : lane < 28u ? a.f_c : 1.0);
+        if (lane == 0) *done = 0u;   // before the fence: a host that sees the serial may launch on another stream
         __threadfence_system();
         __syncwarp();
-        if (lane == 0) {
-            *done = 0u;
-            *reinterpret_cast<volatile double*>(out + 31) = a.serial;   // the system above is complete
-        }
+        if (lane == 0) *reinterpret_cast<volatile double*>(out + 31) = a.serial;   // the system above is complete
     }
 }
 

@@ -90,3 +90,38 @@ def test_first_registration_on_side_stream(n):
             assert np.allclose(g, ref, rtol=1e-9, atol=1e-12 * np.abs(ref).max())
     finally:
         m.close()
+
+
+def test_registration_leaves_its_stream_idle():
+    """A registration synchronises its stream: whatever it returns, the stream has nothing left to do, and the
+    next evaluation may use another one."""
+    from paper_2310_05766_gb300 import binding as b
+    p = synth.params_dict((64, 64, 64), 0.1, 0.3, 64, 0.0, 0.1, 10.0, 0, (-32, -32, -32))
+    g = np.stack(np.meshgrid(*[np.arange(-32, 32) + 0.5] * 3, indexing="ij"), -1)[..., ::-1] * 0.1
+    value = np.rint(np.clip(2.0 - np.linalg.norm(g, axis=-1), -0.3, 0.3) * 32767 / 0.3).astype(np.int16)
+    rng = np.random.default_rng(3)
+    d = rng.normal(size=(20000, 3))
+    pts = np.zeros((20000, 4), np.float32)
+    pts[:, :3] = d / np.linalg.norm(d, axis=1, keepdims=True) * 2.0
+    pose = synth.pose12(synth.rot_zyx(0.01, -0.02, 0.01), np.array([0.02, -0.03, 0.01]))
+    m = b.TsdfMap(p)
+    try:
+        m.write(value, np.ones_like(value))
+        dev = torch.from_numpy(pts).cuda()
+        far = dev + 1000.0
+        streams = [torch.cuda.Stream() for _ in range(2)]
+        ref = b.tsdf_register_system(m.handle, dev, pose)
+        assert ref[28] > 10000
+        for k in range(200):
+            s = streams[k & 1]
+            with torch.cuda.stream(s):
+                got = b.tsdf_register_system(m.handle, dev, pose)
+                assert s.query() and np.array_equal(got, ref)
+                if k % 10 == 0:
+                    with pytest.raises(b.TsdfError):
+                        b.tsdf_register(m.handle, far, pose, iterations=3)
+                    assert s.query()
+                    b.tsdf_register(m.handle, dev, pose, iterations=2)
+                    assert s.query()
+    finally:
+        m.close()
