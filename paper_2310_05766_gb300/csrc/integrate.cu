@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, co
 
 template <bool POOL>
 __device__ __forceinline__ void cache_init(uint32_t* btab) {
-    for (int i = threadIdx.x; i < (POOL ? 2 * kSlotCache : kBrickCache); i += blockDim.x) btab[i] = kNoVoxel;
+    for (int i = threadIdx.x; i < (POOL ? kSlotCacheWords : kBrickCache); i += blockDim.x) btab[i] = kNoVoxel;
 }
 
 // The CTA's cache for a march: of marked bricks, or (pool reduction) of claimed
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
                                                                                         const MapDev m,
                                                                                         const int kpt_max) {
     __shared__ unsigned long long red[kContribThreads / 32];
-    __shared__ __align__(8) uint32_t btab[POOL ? 2 * kSlotCache : kBrickCache];   // POOL: the slot cache
+    __shared__ __align__(8) uint32_t btab[POOL ? kSlotCacheWords : kBrickCache];   // POOL: the slot cache
     const unsigned lane = threadIdx.x & 31u;
     const unsigned gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kScanThreads, TSDF_SCAN_MIN_CTAS) scan_kernel(
                                                                                const int tile, const int parts,
                                                                                const int kpt_max) {
     __shared__ float4 s_a[kScanThreads], s_b[kScanThreads];
-    __shared__ __align__(8) uint32_t btab[POOL ? 2 * kSlotCache : kBrickCache];   // POOL: the slot cache
+    __shared__ __align__(8) uint32_t btab[POOL ? kSlotCacheWords : kBrickCache];   // POOL: the slot cache
     __shared__ unsigned s_heavy[kScanWarps], s_light[kScanWarps], s_valid[kScanWarps];
     __shared__ unsigned s_next;
     __shared__ unsigned long long red[kScanWarps];

@@ -22,9 +22,11 @@ struct BrickCache {
     uint32_t tag = 0;
     unsigned long long* slots = nullptr;   // pool reduction: brick (high word) -> slot, direct mapped
 };
-// Pool reduction: entries of a CTA's slot cache.
+// Pool reduction: entries of a CTA's slot cache; one more word behind them is 0
+// once a claim of the CTA has found the pool full.
 constexpr int kSlotCacheLog2 = 11;
 constexpr int kSlotCache = 1 << kSlotCacheLog2;
+constexpr int kSlotCacheWords = 2 * (kSlotCache + 1);   // 32-bit
 constexpr unsigned long long kNoSlotEntry = ~0ull;
 
 // The per-map contribution kernels keep one cache per CTA.
@@ -361,7 +363,7 @@ __device__ __forceinline__ void load_rays(const MapDev& m, unsigned end, unsigne
 constexpr uint32_t kPoolClaiming = 0xFFFFFFFEu;
 constexpr long long kPoolSpinLimit = 1LL << 20;
 
-__device__ __forceinline__ uint32_t pool_slot(const MapDev& m, unsigned brick) {
+__device__ __forceinline__ uint32_t pool_slot(const MapDev& m, unsigned brick, volatile unsigned long long* full) {
     uint32_t s = __ldcg(m.pool_table + brick);
     if (s < kPoolClaiming) return s;
     const unsigned act = __activemask();
@@ -378,14 +380,20 @@ __device__ __forceinline__ uint32_t pool_slot(const MapDev& m, unsigned brick) {
                     m.pool_brick[ns] = brick;
                     s = ns;
                 } else {
+                    *full = 0ull;
                     atomicExch(&m.ctr->pool_overflow, 1u);
                     atomicExch(m.pool_table + brick, kPoolEmpty);
                 }
                 break;
             }
             // another warp is claiming it
+            if (*full == 0ull) {
+                s = kPoolEmpty;
+                break;
+            }
             if (++spins > kPoolSpinLimit) atomicExch(&m.ctr->pool_overflow, 1u);
             if ((spins & 15) == 0 && __ldcg(&m.ctr->pool_overflow) != 0u) {
+                *full = 0ull;
                 s = kPoolEmpty;
                 break;
             }
@@ -425,12 +433,17 @@ __device__ __forceinline__ void mark_brick(const MapDev& m, unsigned brick, cons
 // the overflow mark before) a 64 x 1024 outdoor scan takes 34 instead of 50 us.
 // Entries are whole 64-bit words, so a reader sees one or another; the
 // table only ever holds claimed slots of this scan, so an entry never goes
-// stale within it.
+// stale within it. Once some lane has found the pool full the CTA claims no
+// more: the scan is dropped, and failing claims would queue up at the counter
+// (64 x 1024 points, a pool of 64: 25 us with the mark, 349 without it)
+// and could in the end carry it round to slots that are taken.
 __device__ __forceinline__ uint32_t cached_pool_slot(const MapDev& m, unsigned brick, const BrickCache& bc) {
     volatile unsigned long long* e = bc.slots + ((brick * 2654435761u) >> (32 - kSlotCacheLog2));
     const unsigned long long v = *e;
     if ((unsigned)(v >> 32) == brick) return (uint32_t)v;
-    const uint32_t s = pool_slot(m, brick);
+    volatile unsigned long long* full = bc.slots + kSlotCache;   // 0: the pool is full
+    if (*full == 0ull) return kPoolEmpty;
+    const uint32_t s = pool_slot(m, brick, full);
     if (s != kPoolEmpty) *e = (unsigned long long)brick << 32 | s;
     return s;
 }
