@@ -443,6 +443,11 @@ const Config kConfigs[] = {
     // 32 served sessions ran at 26 k instead of 30 k scans/s)
     {false, 4, false, 128, 0, kP, kBatchRaysPPT}};
 constexpr int kNumConfigs = 13;
+// CTAs of 128 threads: half a device of them fits beside half a device of any
+// configuration (six per SM). Half a device of 256-thread CTAs does not fit
+// beside one of 128-thread CTAs: three of those leave an SM registers for one
+// of the three per two SMs that are wanted.
+constexpr int kFineConfig = 8;
 
 // Dynamic shared memory of a configuration: the apply staging area (per warp)
 // where the apply stages bricks, else only phase 2's brick caches (one per CTA,
@@ -489,7 +494,7 @@ struct tsdf_batch {
         unsigned char* dev = nullptr;
         cudaEvent_t done = nullptr;        // recorded after the set's launch
         bool pending = false;
-        cudaGraphExec_t exec[2][kNumConfigs] = {};   // by grid (its share of the device, or all of it)
+        cudaGraphExec_t exec[kNumConfigs] = {};
     } slot[2];
     int next_slot = 0;
     BatchSync* sync = nullptr;
@@ -533,9 +538,8 @@ struct DevScope {
 void free_batch(tsdf_batch* b) {
     if (!b) return;
     for (auto& s : b->slot) {
-        for (auto& g : s.exec)
-            for (auto& e : g)
-                if (e) cudaGraphExecDestroy(e);
+        for (auto& e : s.exec)
+            if (e) cudaGraphExecDestroy(e);
         if (s.host) cudaFreeHost(s.host);
         cudaFree(s.dev);
         if (s.done) cudaEventDestroy(s.done);
@@ -550,21 +554,20 @@ void free_batch(tsdf_batch* b) {
 }
 
 // CTAs launched for configuration `cfg`: its co-resident CTAs (limited to
-// ctas_per_sm per SM when set), scaled by the grid-fraction option unless the
-// launch takes the whole device.
-int grid_of(const tsdf_batch* b, int cfg, bool whole = false) {
-    return std::max(1, (int)((long long)b->grid_max[cfg] * (whole ? 100 : b->grid_pct) / 100));
+// ctas_per_sm per SM when set), scaled by the grid-fraction option.
+int grid_of(const tsdf_batch* b, int cfg) {
+    return std::max(1, (int)((long long)b->grid_max[cfg] * b->grid_pct / 100));
 }
 
 // Enqueue copy + barrier reset + cooperative kernel for descriptor slot `si`.
-cudaError_t enqueue(tsdf_batch* b, int si, int cfg, bool whole, cudaStream_t s) {
+cudaError_t enqueue(tsdf_batch* b, int si, int cfg, cudaStream_t s) {
     tsdf_batch::Slot& sl = b->slot[si];
     cudaError_t e = cudaMemcpyAsync(sl.dev, sl.host, b->desc_bytes, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->sync, 0, sizeof(BatchSync), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t lc = {};
     const Config& c = kConfigs[cfg];
-    lc.gridDim = dim3((unsigned)grid_of(b, cfg, whole));
+    lc.gridDim = dim3((unsigned)grid_of(b, cfg));
     lc.blockDim = dim3((unsigned)c.threads);
     lc.dynamicSmemBytes = dyn_smem(c);
     lc.stream = s;
@@ -689,7 +692,7 @@ int tsdf_batch_set_option(tsdf_batch* b, int32_t option, int64_t value) {
                             cudaEventSynchronize(sl.done);
                             sl.pending = false;
                         }
-                        for (auto& e : sl.exec[0])   // (the whole-device graphs stay as they are)
+                        for (auto& e : sl.exec)
                             if (e) {
                                 cudaGraphExecDestroy(e);
                                 e = nullptr;
@@ -740,7 +743,7 @@ int tsdf_batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* cons
 namespace tsdf {
 
 int batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* const* points_dev, const int64_t* n,
-                    const float* poses, int32_t count, bool whole, void* stream) {
+                    const float* poses, int32_t count, bool beside, void* stream) {
     if (!b || !maps || !points_dev || !n || !poses || count < 0 || count > b->max_count) return TSDF_ERR_INVALID;
     if (count == 0) return TSDF_OK;
     for (int i = 0; i < count; ++i) {
@@ -757,10 +760,11 @@ int batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* const* po
         if (e != cudaSuccess) return cu_fail(e);
         sl.pending = false;
     }
-    if (b->autotune && b->tuned < 0) harvest_trials(b);
-    int cfg = b->config;
+    const bool tuning = b->autotune && b->tuned < 0 && !beside;
+    if (tuning) harvest_trials(b);
+    int cfg = beside ? kFineConfig : b->config;
     bool timing = false;
-    if (b->autotune && b->tuned < 0) {
+    if (tuning && b->tuned < 0) {
         // cycle through the configurations until each has been timed enough
         int pending_of[kNumConfigs] = {};
         for (auto& t : b->trials) pending_of[t.config]++;
@@ -809,21 +813,21 @@ int batch_integrate(tsdf_batch* b, tsdf_map* const* maps, const float* const* po
     }
     if (e == cudaSuccess) {
         if (b->use_graph) {
-            if (!sl.exec[whole][cfg]) {
+            if (!sl.exec[cfg]) {
                 // capture copy + reset + kernel once for this slot and config
                 cudaGraph_t g = nullptr;
                 e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal);
                 if (e == cudaSuccess) {
-                    cudaError_t e2 = enqueue(b, si, cfg, whole, b->capture_stream);
+                    cudaError_t e2 = enqueue(b, si, cfg, b->capture_stream);
                     e = cudaStreamEndCapture(b->capture_stream, &g);
                     if (e == cudaSuccess) e = e2;
                 }
-                if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec[whole][cfg], g, 0);
+                if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec[cfg], g, 0);
                 if (g) cudaGraphDestroy(g);
             }
-            if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec[whole][cfg], s);
+            if (e == cudaSuccess) e = cudaGraphLaunch(sl.exec[cfg], s);
         } else {
-            e = enqueue(b, si, cfg, whole, s);
+            e = enqueue(b, si, cfg, s);
         }
     }
     if (e == cudaSuccess && timing) {

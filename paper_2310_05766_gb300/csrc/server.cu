@@ -77,6 +77,7 @@ struct Slot {
     std::vector<const volatile long long*> src;   // per request: where its counters are read
     bool busy = false;
     bool launching = false;             // being filled by the worker outside the lock
+    bool batched = false;               // busy with a batched launch (worker thread only)
 };
 
 // Device-tier slots of a session's global store (rounded up to the 8 MiB
@@ -124,18 +125,13 @@ namespace {
 // (two or three short kernels each) instead of one cooperative batched launch,
 // whose fixed cost (five phases, grid barriers) dominates when it carries only
 // a few scans (three of them: 118 against 141 us): the latency of a lone
-// request is what a lightly loaded server sees.
+// request is what a lightly loaded server sees. Not while another slot runs a
+// batched launch: a plain scan's apply, one large CTA per SM, finds no room
+// beside that launch's CTAs and would wait for its end, while this slot's own
+// share of the device is free. A request 20 us behind a burst of 8 / 16 mixed
+// scans: 126 / 119 us, as plain kernels 262 / 414.
 #ifndef TSDF_SERVER_PLAIN_BATCH
 #define TSDF_SERVER_PLAIN_BATCH 3
-#endif
-
-// Batches of at least this many requests take the whole device when they are
-// alone (nothing in flight on the other slots, nothing left in the queues)
-// instead of the slot's share: a burst of 16 mixed scans 434 against 487 us, of
-// 5 scans 163 against 180. (Smaller ones run as plain integrations, beside
-// which a request that arrives meanwhile can run.)
-#ifndef TSDF_SERVER_WHOLE_BATCH
-#define TSDF_SERVER_WHOLE_BATCH 5
 #endif
 
 void release_request(tsdf_server* s, Request* r) {
@@ -147,7 +143,7 @@ void release_request(tsdf_server* s, Request* r) {
 // slot belong to the worker until it records the launch (`maps` were taken
 // under the lock; sessions in flight cannot be closed).
 int launch_batch(tsdf_server* s, int k, std::vector<Request*>& reqs, const std::vector<tsdf_map*>& smaps,
-                 bool alone) {
+                 bool plain) {
     Slot& sl = s->slots[k];
     const int count = (int)reqs.size();
     std::vector<tsdf_map*> maps(count);
@@ -178,12 +174,13 @@ int launch_batch(tsdf_server* s, int k, std::vector<Request*>& reqs, const std::
     }
     if (e != cudaSuccess) return TSDF_ERR_CUDA;
     int rc = TSDF_OK;
-    if (count <= TSDF_SERVER_PLAIN_BATCH) {
+    sl.batched = !plain;
+    if (plain) {
         for (int i = 0; i < count && rc == TSDF_OK; ++i)
             rc = tsdf_integrate(maps[i], pts[i], ns[i], &poses[12 * (size_t)i], sl.stream);
     } else {
         rc = batch_integrate(sl.batch, maps.data(), pts.data(), ns.data(), poses.data(), count,
-                             alone && count >= TSDF_SERVER_WHOLE_BATCH, sl.stream);
+                             count <= TSDF_SERVER_PLAIN_BATCH, sl.stream);
     }
     if (rc != TSDF_OK) return rc;
     // counters: the mapped host copy the batch writes (no copy to issue), else
@@ -265,14 +262,13 @@ void worker_loop(tsdf_server* s) {
                 ss.in_flight = true;
                 maps.push_back(ss.map);
             }
-            bool alone = true;
-            for (const Slot& other : s->slots) alone = alone && !other.busy;
-            for (auto& kv : s->sessions) alone = alone && kv.second.queue.empty();
+            bool plain = (int)reqs.size() <= TSDF_SERVER_PLAIN_BATCH;
+            for (const Slot& other : s->slots) plain = plain && !(other.busy && other.batched);
             Slot& sl = s->slots[k];
             sl.busy = true;
             sl.launching = true;
             lk.unlock();
-            int rc = launch_batch(s, (int)k, reqs, maps, alone);
+            int rc = launch_batch(s, (int)k, reqs, maps, plain);
             lk.lock();
             sl.launching = false;
             if (rc == TSDF_OK) {

@@ -197,10 +197,11 @@ int map_reserve_points(::tsdf_map* map, int64_t n);
 // (synchronous allocation on first use or growth).
 int map_reserve_sort(::tsdf_map* map, int64_t n);
 
-// tsdf_batch_integrate; whole: on all of the device whatever the batch's grid
-// fraction.
+// tsdf_batch_integrate; beside: a small launch that has to run beside another
+// batch object's share of the device (in the shape that fits beside any, and
+// without a say in the autotuner's choice).
 int batch_integrate(::tsdf_batch* batch, ::tsdf_map* const* maps, const float* const* points_dev, const int64_t* n,
-                    const float* poses, int32_t count, bool whole, void* stream);
+                    const float* poses, int32_t count, bool beside, void* stream);
 
 // Launchers (return the cudaError_t of the launch).
 // Ray set-up into the map's ray list. sort: pair slots per ray too (sort

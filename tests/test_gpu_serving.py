@@ -233,3 +233,42 @@ def test_serving_config_shapes_equal_oracle():
         assert b.tsdf_server_get_stats(srv)["mean_batch"] > 1.0
     finally:
         b.tsdf_server_destroy(srv)
+
+
+def test_request_behind_a_burst_overlaps_it():
+    """A small request that arrives while a large batch is on the device runs beside it on the other stream and is
+    done before the batch; the maps are the same as alone."""
+    from paper_2310_05766_gb300 import binding as b
+    ws = [synth.workload_outdoor(n_scans=1, seed=700 + i, beams=128, azimuths=2048) for i in range(2)]
+    small = synth.workload_outdoor(n_scans=1, seed=710, beams=16, azimuths=1024)
+    srv = b.tsdf_server_create(hbm_budget_bytes=64 << 30, max_points=1 << 18, max_batch=32, streams=2,
+                               max_outstanding=64)
+    try:
+        sids = [b.tsdf_server_open_session(srv, ws[i % 2].params) for i in range(16)]
+        lone = b.tsdf_server_open_session(srv, small.params)
+        pin = [torch.from_numpy(np.ascontiguousarray(w.scans[0], np.float32)).pin_memory() for w in [*ws, small]]
+        poses = np.stack([ws[i % 2].poses[0] for i in range(16)])
+        passes, before = 60, 0
+        for _ in range(passes):
+            tk = b.tsdf_server_submit_many(srv, sids, [pin[i % 2] for i in range(16)], poses)
+            assert len(tk) == 16
+            while b.tsdf_server_get_stats(srv)["queued"]:
+                pass
+            one = b.tsdf_server_submit(srv, lone, pin[2], small.poses[0])
+            r = b.tsdf_server_wait(srv, one)
+            done = max(x["t_done_us"] for x in b.tsdf_server_wait_many(srv, tk))
+            before += r["t_done_us"] < done
+        assert before > passes // 2, (before, passes)
+        for w, sid in [(ws[0], sids[0]), (ws[1], sids[1]), (small, lone)]:
+            m = b.TsdfMap(w.params)
+            pts = torch.from_numpy(np.ascontiguousarray(w.scans[0], np.float32)).cuda()
+            for _ in range(passes):
+                m.integrate(pts, w.poses[0])
+            v, wt = m.read()
+            m.close()
+            mh = b.tsdf_server_session_map(srv, sid)
+            o, d = b.tsdf_get_origin(mh), w.params["dims"]
+            vs, wts = b.tsdf_read(mh, o, tuple(o[a] + d[a] for a in range(3)))
+            assert np.array_equal(v, vs) and np.array_equal(wt, wts)
+    finally:
+        b.tsdf_server_destroy(srv)
