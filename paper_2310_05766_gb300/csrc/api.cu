@@ -134,7 +134,7 @@ struct tsdf_map {
     bool pdl = true;                // programmatic dependent launch between the scan's kernels
     int reduction = TSDF_REDUCTION_ATOMIC;   // per-scan reduction: accumulator atomics or sort
     bool zero_copy = true;          // tsdf_integrate_host reads device-mapped pinned points in place
-    // The plain path's launches as one CUDA graph (TSDF_OPT_LAUNCH_GRAPH):
+    // The plain path's launches as a CUDA graph (TSDF_OPT_LAUNCH_GRAPH):
     // captured on first use, then per scan the ray and contribution nodes get
     // the scan's arguments and the graph is launched once. Off by default: it
     // cuts the host's time per scan from about 9 to 3.5 us, but back-to-back
@@ -143,17 +143,18 @@ struct tsdf_map {
     bool use_graph = false;
     bool graph_broken = false;      // capture or instantiation failed: plain launches from then on
     cudaStream_t capture_stream = nullptr;
-    cudaGraph_t chain_graph = nullptr;
-    cudaGraphExec_t chain_exec = nullptr;
-    cudaGraphNode_t node_rays = nullptr;
-    cudaGraphNode_t node_contrib = nullptr;
-    cudaKernelNodeParams kp_rays{};
-    cudaKernelNodeParams kp_contrib{};
-    bool chain_fused = false;
-    MapDev chain_dev{};             // the buffers and options the graph was captured with
-    int chain_kpt = 0;
-    bool chain_merge = false;
-    bool chain_pdl = false;
+    struct ScanGraph {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t exec = nullptr;
+        cudaGraphNode_t node_rays = nullptr;
+        cudaGraphNode_t node_contrib = nullptr;
+        cudaKernelNodeParams kp_rays{};
+        cudaKernelNodeParams kp_contrib{};
+        MapDev dev{};               // the buffers and options the graph was captured with
+        int kpt = 0;
+        bool merge = false;
+        bool pdl = false;
+    } chain[2];                     // of larger scans and of one-kernel ones (scan_fused): a map may see both by turns
     long long* host_last = nullptr; // mapped pinned copy of the published counters (host address)
     double* reg_dev = nullptr;      // registration: the CTAs' sums, the 29 sums of the normal equations, a counter
     double reg_serial = 0.0;        // registration: evaluations so far
@@ -258,17 +259,15 @@ int prof_drain(tsdf_map* m) {
     return TSDF_OK;
 }
 
-static void chain_graph_reset(tsdf_map* m) {
-    if (m->chain_exec) cudaGraphExecDestroy(m->chain_exec);
-    if (m->chain_graph) cudaGraphDestroy(m->chain_graph);
-    m->chain_exec = nullptr;
-    m->chain_graph = nullptr;
-    m->node_rays = m->node_contrib = nullptr;
+static void chain_graph_reset(tsdf_map::ScanGraph& c) {
+    if (c.exec) cudaGraphExecDestroy(c.exec);
+    if (c.graph) cudaGraphDestroy(c.graph);
+    c = tsdf_map::ScanGraph{};
 }
 
 void free_map(tsdf_map* m) {
     if (!m) return;
-    chain_graph_reset(m);
+    for (auto& c : m->chain) chain_graph_reset(c);
     if (m->capture_stream) cudaStreamDestroy(m->capture_stream);
     for (const Pending& p : m->pending) {
         cudaEventDestroy(p.start);
@@ -747,10 +746,10 @@ static bool same_dev(const MapDev& x, const MapDev& y) {
 }
 
 // Capture the plain atomic path (scan or rays + contribution, apply with
-// the map's options) into chain_graph and instantiate it; false when any step
-// fails (nothing is left half built).
-static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
-    chain_graph_reset(map);
+// the map's options) into the graph `c` of its form and instantiate it; false
+// when any step fails (nothing is left half built).
+static bool chain_graph_build(tsdf_map* map, tsdf_map::ScanGraph& c, const ScanArgs& a) {
+    chain_graph_reset(c);
     if (!map->capture_stream &&
         cudaStreamCreateWithFlags(&map->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
         map->capture_stream = nullptr;
@@ -797,27 +796,26 @@ static bool chain_graph_build(tsdf_map* map, const ScanArgs& a) {
         if (cudaGraphNodeGetType(node, &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
         if (cudaGraphKernelNodeGetParams(node, &kp) != cudaSuccess) continue;
         if (kp.func == fr) {
-            map->node_rays = node;
-            map->kp_rays = kp;
+            c.node_rays = node;
+            c.kp_rays = kp;
         } else if (kp.func == fc) {
-            map->node_contrib = node;
-            map->kp_contrib = kp;
+            c.node_contrib = node;
+            c.kp_contrib = kp;
         }
     }
     cudaGraphExec_t x = nullptr;
-    if ((!fused && !map->node_rays) || !map->node_contrib || cudaGraphInstantiate(&x, g, 0) != cudaSuccess) {
-        map->node_rays = map->node_contrib = nullptr;
+    if ((!fused && !c.node_rays) || !c.node_contrib || cudaGraphInstantiate(&x, g, 0) != cudaSuccess) {
+        c.node_rays = c.node_contrib = nullptr;
         cudaGraphDestroy(g);
         cudaGetLastError();
         return false;
     }
-    map->chain_graph = g;
-    map->chain_exec = x;
-    map->chain_dev = map->dev;
-    map->chain_kpt = map->kpt;
-    map->chain_merge = map->merge;
-    map->chain_pdl = map->pdl;
-    map->chain_fused = fused;
+    c.graph = g;
+    c.exec = x;
+    c.dev = map->dev;
+    c.kpt = map->kpt;
+    c.merge = map->merge;
+    c.pdl = map->pdl;
     return true;
 }
 
@@ -833,11 +831,11 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
         return TSDF_OK;
     }
     if (cap != cudaStreamCaptureStatusNone) return TSDF_OK;
-    if (map->chain_exec && (!same_dev(map->chain_dev, map->dev) ||
-                            map->chain_kpt != map->kpt || map->chain_merge != map->merge ||
-                            map->chain_pdl != map->pdl || map->chain_fused != scan_fused(a.n)))
-        chain_graph_reset(map);
-    if (!map->chain_exec && !chain_graph_build(map, a)) {
+    const bool fused = scan_fused(a.n);
+    tsdf_map::ScanGraph& c = map->chain[fused];
+    if (c.exec && (!same_dev(c.dev, map->dev) || c.kpt != map->kpt || c.merge != map->merge || c.pdl != map->pdl))
+        chain_graph_reset(c);
+    if (!c.exec && !chain_graph_build(map, c, a)) {
         map->graph_broken = true;
         return TSDF_OK;
     }
@@ -846,27 +844,27 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
     d.parity = 0;
     void* fused_args[5] = {const_cast<ScanArgs*>(&a), &d, &g.tile, &g.parts, &map->kpt};
     void* list_args[3] = {const_cast<ScanArgs*>(&a), &d, &map->kpt};   // (the ray set-up takes the first two)
-    cudaKernelNodeParams kc = map->kp_contrib;
-    kc.kernelParams = map->chain_fused ? fused_args : list_args;
+    cudaKernelNodeParams kc = c.kp_contrib;
+    kc.kernelParams = fused ? fused_args : list_args;
     kc.extra = nullptr;
-    if (map->chain_fused) kc.gridDim = dim3(g.grid);
-    cudaError_t e = cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_contrib, &kc);
-    if (e == cudaSuccess && !map->chain_fused) {
-        cudaKernelNodeParams kr = map->kp_rays;
+    if (fused) kc.gridDim = dim3(g.grid);
+    cudaError_t e = cudaGraphExecKernelNodeSetParams(c.exec, c.node_contrib, &kc);
+    if (e == cudaSuccess && !fused) {
+        cudaKernelNodeParams kr = c.kp_rays;
         kr.gridDim = dim3(rays_grid(a.n, false));
         kr.kernelParams = list_args;
         kr.extra = nullptr;
-        e = cudaGraphExecKernelNodeSetParams(map->chain_exec, map->node_rays, &kr);
+        e = cudaGraphExecKernelNodeSetParams(c.exec, c.node_rays, &kr);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
-        chain_graph_reset(map);
+        chain_graph_reset(c);
         map->graph_broken = true;
         return TSDF_OK;
     }
     *launched = true;
     map->dev.parity = 0;   // (the next plain scan takes the other set)
-    TSDF_CU(cudaGraphLaunch(map->chain_exec, s));
+    TSDF_CU(cudaGraphLaunch(c.exec, s));
     return TSDF_OK;
 }
 
