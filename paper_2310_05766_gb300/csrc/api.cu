@@ -142,6 +142,7 @@ struct tsdf_map {
     // overlap of one scan's last kernel with the next scan's first is lost).
     bool use_graph = false;
     bool graph_broken = false;      // capture or instantiation failed: plain launches from then on
+    bool captured = false;          // a caller has captured a plain scan of this map (see note_capture)
     cudaStream_t capture_stream = nullptr;
     struct ScanGraph {
         cudaGraph_t graph = nullptr;
@@ -735,7 +736,7 @@ static void fill_scan_args(const tsdf_map* map, const float* points_dev, int64_t
     fill_lean_args(a);
 }
 
-static_assert(sizeof(MapDev) == 168, "same_dev compares every field of MapDev but the parity");
+static_assert(sizeof(MapDev) == 168, "same_dev compares every field of MapDev but parity and wait_first");
 static bool same_dev(const MapDev& x, const MapDev& y) {
     return x.grid == y.grid && x.acc == y.acc && x.brick_flag == y.brick_flag && x.brick_list == y.brick_list &&
            x.ray_a == y.ray_a && x.ray_b == y.ray_b && x.ray_cap == y.ray_cap && x.ctr == y.ctr &&
@@ -762,7 +763,8 @@ static bool chain_graph_build(tsdf_map* map, tsdf_map::ScanGraph& c, const ScanA
         return false;
     }
     MapDev d = map->dev;
-    d.parity = 0;   // graph launches do not overlap: the graph's nodes keep one set of ray counts
+    d.parity = 0;       // the graph's nodes keep one set of ray counts
+    d.wait_first = 1;   // (so they count when the previous scan is over)
     const bool fused = scan_fused(a.n);
     cudaError_t e = cudaSuccess;
     if (fused) {
@@ -842,6 +844,7 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
     ScanShape g = scan_shape(a.n, a.K);
     MapDev d = map->dev;
     d.parity = 0;
+    d.wait_first = 1;
     void* fused_args[5] = {const_cast<ScanArgs*>(&a), &d, &g.tile, &g.parts, &map->kpt};
     void* list_args[3] = {const_cast<ScanArgs*>(&a), &d, &map->kpt};   // (the ray set-up takes the first two)
     cudaKernelNodeParams kc = c.kp_contrib;
@@ -866,6 +869,21 @@ static int chain_graph_launch(tsdf_map* map, const ScanArgs& a, cudaStream_t s, 
     map->dev.parity = 0;   // (the next plain scan takes the other set)
     TSDF_CU(cudaGraphLaunch(c.exec, s));
     return TSDF_OK;
+}
+
+// Whether a caller has captured a plain scan of this map into a graph of its
+// own. Such a scan keeps the ray counts that it was captured with (parity), in
+// whatever order it is replayed among direct calls, so from then on the map's
+// ray set-up waits for the previous scan before it counts.
+static bool note_capture(tsdf_map* map, cudaStream_t s) {
+    if (map->captured) return true;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        st = cudaStreamCaptureStatusActive;
+    }
+    map->captured = st != cudaStreamCaptureStatusNone;
+    return map->captured;
 }
 
 static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, const float pose[12], cudaStream_t s,
@@ -914,6 +932,7 @@ static int integrate_with(tsdf_map* map, const float* points_dev, int64_t n, con
         if (launched || rc != TSDF_OK) return rc;
     }
     map->dev.parity ^= 1u;   // this scan's ray counts (see LiveCounts)
+    map->dev.wait_first = note_capture(map, s) ? 1u : 0u;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (!fused) {
         e0 = prof_mark(map, s);

@@ -244,8 +244,8 @@ constexpr int kBatchRaysPPT = TSDF_BATCH_RAYS_PPT;
 // which are over when this kernel starts (every apply kernel triggers its
 // dependents after its own wait): so nothing here waits for the previous scan,
 // and the set-up runs beside its apply (the kernel's first CTA waits before it
-// ends, so that what follows sees that scan complete).
-// Otherwise, with PDL, the wait comes before the map's counters and ray list.
+// ends, so that what follows sees that scan complete). With wait_first (scans in
+// graphs, which do not alternate their parity) every CTA waits first.
 template <bool PDL, bool SPLIT, int NW, int PPT>
 __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m, int base, unsigned part,
                                               RaysSmemT<NW>* sm) {
@@ -294,7 +294,7 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
         if (SPLIT) sm->ws[warp] = wf;
     }
     __syncthreads();
-    if (PDL && !SPLIT) pdl_wait();   // the previous scan's finish resets live_count and the counters
+    if (PDL && SPLIT && m.wait_first) pdl_wait();
     if (threadIdx.x == 0) {
         unsigned tl = 0, tv = 0, tb = 0, tf = 0;
         for (int w = 0; w < NW; ++w) {

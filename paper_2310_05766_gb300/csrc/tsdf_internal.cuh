@@ -84,7 +84,7 @@ struct MapDev {
     MapCounters* ctr;
     long long* host_last;           // mapped pinned host memory for the published counters (kPubWords), or null
     uint32_t parity;                // which LiveCounts the plain scan in flight uses
-    uint32_t pad_;
+    uint32_t wait_first;            // 1: its ray set-up counts only when the previous scan is over (graphs)
     // sort reduction (null / 0 when the map has no sort buffers)
     uint32_t* brick_slot;           // per brick: its position in the brick list (touched bricks only)
     uint32_t* seg_count;            // per list position: pair count, then the scatter cursor; zero between scans

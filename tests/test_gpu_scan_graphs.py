@@ -60,3 +60,43 @@ def test_launch_graph_alternating_sizes(reduce):
         assert host_us([3, 4] * 10) < 3 * same
     finally:
         m.close()
+
+
+@pytest.mark.parametrize("sizes", [[40000, 60000, 50000], [2000, 60000, 40000], [60000, 3000, 32769]])
+def test_captured_scans_mixed_with_direct_calls(sizes):
+    """Scans captured into the caller's graphs, one and three at a time, replayed in any order among direct calls:
+    the same map as the scans in that order."""
+    from paper_2310_05766_gb300 import binding as b
+    p, scans, poses = _case(sizes)
+    m = b.TsdfMap(p)
+    try:
+        dev = [torch.from_numpy(s).cuda() for s in scans]
+        order = []
+
+        def direct(i):
+            m.integrate(dev[i], poses[i])
+            order.append(i)
+
+        for i in range(3):
+            direct(i)
+        m.stats()
+        graphs = []
+        for ids in ([0], [1], [0, 1, 2]):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                for i in ids:
+                    m.integrate(dev[i], poses[i])
+            graphs.append((g, ids))
+        rng = np.random.default_rng(sum(sizes))
+        for k in rng.integers(0, 6, 24):
+            if k < 3:
+                graphs[k][0].replay()
+                order.extend(graphs[k][1])
+            else:
+                direct(int(k) - 3)
+        stats = m.stats()
+        v, w = m.read()
+        ref = run_oracle(p, [("scan", scans[i], poses[i]) for i in order])
+        assert_same((v, w, [stats], m.origin), (ref[0], ref[1], ref[2][-1:], ref[3]))
+    finally:
+        m.close()
