@@ -277,7 +277,7 @@ int tsdf_stats(tsdf_map* map, tsdf_scan_stats* out, void* stream);
                                     one launch per kernel. */
 
 /* Device memory held by the map (grid, per-scan buffers of the reductions
- * that have been used, ray buffers, global store) in bytes. Host-side.
+ * that have been used, ray buffers, registration, global store) in bytes. Host-side.
  * Errors: INVALID. */
 int tsdf_map_device_bytes(const tsdf_map* map, int64_t* out);
 

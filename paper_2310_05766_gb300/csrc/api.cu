@@ -1603,15 +1603,17 @@ int tsdf_extract_mesh(tsdf_map* map, int32_t min_weight, float* out_dev, int64_t
 // How long a registration watches for an evaluation's sums before it blocks (an
 // evaluation of 2^17 points takes 30 us).
 constexpr int kRegisterWatchUs = 200;
+constexpr size_t kRegisterBytes = ((size_t)kRegisterMaxCtas * 32 + 32 + 1) * sizeof(double);
 
 // Registration buffers, on first use: kRegisterMaxCtas x 32 sums, the system
 // (where no mapped host memory could be had) and the arrival counter.
 static int ensure_register(tsdf_map* map) {
     if (map->reg_dev) return TSDF_OK;
     constexpr size_t kSums = (size_t)kRegisterMaxCtas * 32;
+    static_assert(kRegisterBytes == (kSums + 32 + 1) * sizeof(double), "sums, system, counter");
     double* d = nullptr;
-    TSDF_CU(cudaMalloc(&d, (kSums + 32 + 1) * sizeof(double)));
-    cudaError_t e = fill_new(d, 0, (kSums + 32 + 1) * sizeof(double));
+    TSDF_CU(cudaMalloc(&d, kRegisterBytes));
+    cudaError_t e = fill_new(d, 0, kRegisterBytes);
     if (e != cudaSuccess) {
         cudaFree(d);
         return cuda_fail(e);
@@ -1758,6 +1760,7 @@ int tsdf_map_device_bytes(const tsdf_map* map, int64_t* out) {
     if (map->dev.pool_table)
         b += map->bricks * sizeof(uint32_t) +
              (size_t)map->dev.pool_cap * (sizeof(uint32_t) + kBrickVoxels * sizeof(unsigned long long));
+    if (map->reg_dev) b += kRegisterBytes;
     b += map->store_seg[0].size() * (size_t)kSegChunks * kChunkBytes;   // the host tier is host memory
     b += map->stage_cap * sizeof(float4) + (map->items_dev ? (map->items_dev_cap + 1) * sizeof(ShiftItem) : 0) +
          map->spill_cap * sizeof(ChunkCopy);

@@ -125,3 +125,21 @@ def test_registration_leaves_its_stream_idle():
                     assert s.query()
     finally:
         m.close()
+
+
+def test_device_bytes_count_registration():
+    """What a map's first registration allocates on the device is in tsdf_map_device_bytes."""
+    from paper_2310_05766_gb300 import binding as b
+    p = synth.params_dict((64, 64, 64), 0.1, 0.3, 64, 0.0, 0.1, 10.0, 0, (-32, -32, -32))
+    m = b.TsdfMap(p)
+    try:
+        before = b.tsdf_map_device_bytes(m.handle)
+        pts = torch.zeros((100, 4), device="cuda")
+        pose = synth.pose12(np.eye(3), np.zeros(3))
+        b.tsdf_register_system(m.handle, pts, pose)
+        after = b.tsdf_map_device_bytes(m.handle)
+        assert after >= before + 512 * 32 * 8
+        b.tsdf_register_system(m.handle, pts, pose)
+        assert b.tsdf_map_device_bytes(m.handle) == after
+    finally:
+        m.close()
