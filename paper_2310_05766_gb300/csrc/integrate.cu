@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     const unsigned lane = threadIdx.x & 31u;
     const unsigned gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    __shared__ unsigned s_counts[3];
+    __shared__ unsigned s_counts[3];   // rays from the front, from the end, steps per item
     pdl_trigger();
     cache_init<POOL>(btab);
     pdl_wait();   // ray list and live count come from the rays kernel
@@ -172,24 +172,32 @@ __global__ void __launch_bounds__(kContribThreads, TSDF_CONTRIB_MIN_CTAS) contri
     // light ones from the end): the blocks of the front come first, so the
     // costly items are taken by the first wave of CTAs and the CTAs that start
     // late get light ones.
-    if (threadIdx.x == 0) {
-        s_counts[0] = __ldcg(&m.ctr->live[m.parity].front);
-        s_counts[1] = __ldcg(&m.ctr->live[m.parity].back);
-        s_counts[2] = __ldcg(&m.ctr->live[m.parity].fill);
-    }
-    __syncthreads();   // (also orders the brick cache initialisation)
-    const unsigned nf = s_counts[0], nb = s_counts[1];
-    const unsigned bf = (nf + 31u) / 32u, bb = (nb + 31u) / 32u;
-    const unsigned steps = (unsigned)(2 * a.K + 1);
     // Steps per item: an item of long steps (high fill columns) is cut while the
     // items are too few to even out over the warps. A 33 k-point corridor scan
     // of 18 lines (some hundred samples a step): 52 -> 28 us; corridor 64x1024
     // 24.6 -> 23.2, outdoor 64x1024 19.1 -> 18.4. Items of short steps stay
     // whole (one of 256^3 voxels at 0.1 m, no fill: 10.5 us with four steps, 12.3
     // with one), as do those of larger scans (corridor 128x2048: 29.2 and 33.3).
-    const float per_step = 1.f + 2.f * (float)s_counts[2] / (float)max(nf + nb, 1u);   // samples of a mean ray
-    int kpt = kpt_max;
-    while (kpt > 1 && (float)kpt * per_step > 14.f && (bf + bb) * ((steps + kpt - 1) / kpt) < 2u * nwarps) kpt >>= 1;
+    // By one thread and without divisions: after an L2 flush, with the kernel's
+    // code out of cache too, each line of it counts (outdoor 128x1024: 17.6 us,
+    // done by every warp with divisions 17.8, the march a second time for a
+    // constant four steps 17.6, only that march and no choice 17.1).
+    const unsigned steps = (unsigned)(2 * a.K + 1);
+    if (threadIdx.x == 0) {
+        const unsigned f = __ldcg(&m.ctr->live[m.parity].front), b = __ldcg(&m.ctr->live[m.parity].back);
+        const unsigned fill = __ldcg(&m.ctr->live[m.parity].fill);
+        const unsigned blocks = (f + 31u) / 32u + (b + 31u) / 32u;
+        const float rays = (float)(f + b), samples = rays + 2.f * (float)fill;   // of one step
+        unsigned k = (unsigned)kpt_max;   // 1, 2 or 4
+        while (k > 1u && (float)k * samples > 14.f * rays && blocks * ((steps + k - 1u) >> (k >> 1)) < 2u * nwarps) k >>= 1;
+        s_counts[0] = f;
+        s_counts[1] = b;
+        s_counts[2] = k;
+    }
+    __syncthreads();   // (also orders the brick cache initialisation)
+    const unsigned nf = s_counts[0], nb = s_counts[1];
+    const unsigned bf = (nf + 31u) / 32u, bb = (nb + 31u) / 32u;
+    const int kpt = (int)s_counts[2];
     const unsigned ngrp = (steps + kpt - 1) / kpt;
     const unsigned nitems = (bf + bb) * ngrp;
     // first ray of block `blk` and the end of its part of the list
