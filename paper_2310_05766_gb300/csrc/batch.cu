@@ -214,11 +214,10 @@ __global__ void __launch_bounds__(THREADS, 768 / THREADS) batch_kernel(const Bat
             p1_map = i;
         }
         if constexpr (SORT)
-            rays_task_sort<false, kBatchWarps>(s_args[0], s_dev[0], (int)((t - hdr->ray_prefix[i]) * THREADS),
-                                                       t, &rsm);
+            rays_task_sort<false, kBatchWarps>(s_args[0], s_dev[0], (int)((t - hdr->ray_prefix[i]) * THREADS), t, &rsm);
         else
-            rays_task_ppt<false, false, kBatchWarps, RPPT>(s_args[0], s_dev[0],
-                                                           (int)((t - hdr->ray_prefix[i]) * THREADS * RPPT), t, &rsm);
+            rays_task_ppt<false, kBatchWarps, RPPT>(s_args[0], s_dev[0],
+                                                    (int)((t - hdr->ray_prefix[i]) * THREADS * RPPT), t, &rsm);
         __syncthreads();
     }
     if (!grid_barrier(sync, arrivals, spin)) return;

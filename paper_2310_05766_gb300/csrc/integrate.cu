@@ -40,8 +40,8 @@
 //   accumulators reset. Each CTA publishes its share of the scan's counters:
 //   touched voxels and, in WSUM mode, the contributions too (the sum of the
 //   decoded weights).
-// finish (the other reductions): the last apply CTA to retire sums the
-//   per-scan counters into the published ones and clears the per-scan state.
+// finish (sort reduction): the last apply CTA to retire sums the per-scan
+//   counters into the published ones and clears the per-scan state.
 //
 // Sort reduction (an alternative to the accumulator atomics, same results):
 // rays also reserve each live ray's pair slots (one per march sample); emit is
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(kRaysThreads) rays_kernel(const ScanArgs a, co
     if constexpr (SORT)
         rays_task_sort<true, kRaysThreads / 32>(a, m, (int)(blockIdx.x * blockDim.x), blockIdx.x, &sm);
     else
-        rays_task_ppt<true, true, kRaysThreads / 32, kRaysPPT>(a, m, (int)(blockIdx.x * blockDim.x) * kRaysPPT,
+        rays_task_ppt<true, kRaysThreads / 32, kRaysPPT>(a, m, (int)(blockIdx.x * blockDim.x) * kRaysPPT,
                                                                 blockIdx.x, &sm);
 }
 
@@ -418,7 +418,7 @@ __global__ void __launch_bounds__(256) compact_kernel(const MapDev m, const uint
     compact_words(m, blockIdx.x * blockDim.x + threadIdx.x, nwords);
 }
 
-constexpr int kApplyWarps = 4;   // CTA size of the sort and pool apply kernels
+constexpr int kApplyWarps = 4;   // CTA size of the sort reduction's apply kernel
 
 // ---- apply of the plain path: one CTA per SM.
 //
@@ -737,7 +737,6 @@ __global__ void __launch_bounds__(kApplyWarps * 32) sort_apply_kernel(const MapD
     }
     finish_if_last(m, &s_last);
 }
-
 
 // Launch with `smem` bytes of dynamic shared memory, with programmatic stream
 // serialisation when `pdl` is set.

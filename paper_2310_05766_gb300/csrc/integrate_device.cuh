@@ -27,7 +27,6 @@ struct BrickCache {
 constexpr int kSlotCacheLog2 = 11;
 constexpr int kSlotCache = 1 << kSlotCacheLog2;
 constexpr int kSlotCacheWords = 2 * (kSlotCache + 1);   // 32-bit
-constexpr unsigned long long kNoSlotEntry = ~0ull;
 
 // The per-map contribution kernels keep one cache per CTA.
 constexpr int kBrickCacheLog2 = 11;
@@ -38,7 +37,6 @@ constexpr int kBrickCache = 1 << kBrickCacheLog2;
 __device__ __forceinline__ void brick_cache_init(uint32_t* btab) {
     for (int i = threadIdx.x; i < kBrickCache; i += blockDim.x) btab[i] = kNoVoxel;
 }
-
 
 __device__ __forceinline__ float fm(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fa(float a, float b) { return __fadd_rn(a, b); }
@@ -230,12 +228,12 @@ __device__ __forceinline__ void rays_task_sort(const ScanArgs& a, const MapDev& 
 constexpr int kRaysPPT = TSDF_RAYS_PPT;
 constexpr int kBatchRaysPPT = TSDF_BATCH_RAYS_PPT;
 
-// The plain path's ray set-up with PPT consecutive points per thread: the
-// CTA's threads set up points [base, base + 32 NW PPT), thread t the points
+// The atomic and pool reductions' ray set-up with PPT consecutive points per
+// thread: the CTA's threads set up points [base, base + 32 NW PPT), thread t the points
 // base + PPT t .. base + PPT t + PPT - 1, whose loads are all in flight at
 // once, and append the live ones (in point order) to the map's ray list with
 // one list atomic per CTA and list end.
-// SPLIT (the per-map plain path): the rays whose fill reaches at least one
+// PLAIN (the per-map kernel, with programmatic dependent launch): the rays whose fill reaches at least one
 // voxel each side at the hit (delta_z r >= vs, the costly ones) go to the
 // front of the list and the others to its end (entry ray_cap - 1 - j for the
 // j-th), so that the contribution kernel can take the costly work first; with
@@ -246,7 +244,7 @@ constexpr int kBatchRaysPPT = TSDF_BATCH_RAYS_PPT;
 // and the set-up runs beside its apply (the kernel's first CTA waits before it
 // ends, so that what follows sees that scan complete). With wait_first (scans in
 // graphs, which do not alternate their parity) every CTA waits first.
-template <bool PDL, bool SPLIT, int NW, int PPT>
+template <bool PLAIN, int NW, int PPT>
 __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m, int base, unsigned part,
                                               RaysSmemT<NW>* sm) {
     const unsigned lane = threadIdx.x & 31u;
@@ -258,7 +256,7 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
         p[k] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i0 + k < a.n) p[k] = __ldg(a.pts + i0 + k);
     }
-    if (PDL) pdl_trigger();
+    if (PLAIN) pdl_trigger();
     float4 ra[PPT], rb[PPT];
     unsigned hv = 0, lv = 0;   // bit k: point k is a live heavy (front) / light (end) ray
     unsigned cv = 0;           // valid rays
@@ -268,8 +266,8 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
         bool valid, live;
         ray_setup(a, p[k], i0 + k < a.n, ra[k], rb[k], valid, live);
         const float fill = live && rb[k].w != 0.f ? fm(fm(a.dz, ra[k].w), a.inv_vs) : 0.f;
-        const bool heavy = !SPLIT || fill >= 1.f;
-        if (SPLIT) cf += (unsigned)fminf(fill, 255.f);
+        const bool heavy = !PLAIN || fill >= 1.f;
+        if (PLAIN) cf += (unsigned)fminf(fill, 255.f);
         if (live && heavy) hv |= 1u << k;
         if (live && !heavy) lv |= 1u << k;
         cv += valid ? 1u : 0u;
@@ -286,15 +284,15 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
         }
     }
     const unsigned wv = __reduce_add_sync(kFull, cv);
-    const unsigned wf = SPLIT ? __reduce_add_sync(kFull, cf) : 0u;
+    const unsigned wf = PLAIN ? __reduce_add_sync(kFull, cf) : 0u;
     if (lane == 31) {
         sm->wl[warp] = il;
         sm->wb[warp] = ib;
         sm->wv[warp] = wv;
-        if (SPLIT) sm->ws[warp] = wf;
+        if (PLAIN) sm->ws[warp] = wf;
     }
     __syncthreads();
-    if (PDL && SPLIT && m.wait_first) pdl_wait();
+    if (PLAIN && m.wait_first) pdl_wait();
     if (threadIdx.x == 0) {
         unsigned tl = 0, tv = 0, tb = 0, tf = 0;
         for (int w = 0; w < NW; ++w) {
@@ -304,9 +302,9 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
             sm->wb[w] = tb;
             tb += b;
             tv += sm->wv[w];
-            if (SPLIT) tf += sm->ws[w];
+            if (PLAIN) tf += sm->ws[w];
         }
-        if (SPLIT) {
+        if (PLAIN) {
             LiveCounts* lc = &m.ctr->live[m.parity];
             sm->base = tl ? atomicAdd(&lc->front, tl) : 0u;
             sm->bbase = tb ? atomicAdd(&lc->back, tb) : 0u;
@@ -332,7 +330,7 @@ __device__ __forceinline__ void rays_task_ppt(const ScanArgs& a, const MapDev& m
             ++off_b;
         }
     }
-    if (PDL && SPLIT && blockIdx.x == 0) pdl_wait();
+    if (PLAIN && blockIdx.x == 0) pdl_wait();
 }
 
 // ---- contrib: rays of one 32-ray block (one per lane, dead lanes r = -1);
@@ -346,12 +344,6 @@ __device__ __forceinline__ void load_rays(const MapDev& m, unsigned end, unsigne
     }
 }
 
-// One warp: the steps of k-group `grp` (kpt steps) of its 32 rays.
-// SORT (sort reduction, MERGE off): each sample of a lane's ray is written to
-// the ray's pair slot sslot + (its index in the ray's march) instead of being
-// reduced: (voxel word, code) inside the window, kNoVoxel outside. Samples
-// whose slot is at or beyond the capacity (or whose ray has none) take the
-// accumulator reduction instead and set `ovf`.
 // Pool reduction: slot of `brick` in the map's pool, claimed on first touch.
 // Lanes of the active set that need the same brick share one claim (match).
 // The claimer moves the brick's table entry from empty to a "claiming" mark
@@ -470,8 +462,8 @@ constexpr uint32_t kMagicBits = 0x4B400000u;   // bit pattern of 1.5 * 2^23
 // What a sample of the lean march reads of its scan and map, as values: the
 // batched kernel keeps both in shared memory, where every store to the brick
 // cache would have them read again sample by sample; a march copies them into
-// registers once. (The per-map kernels have them in constant memory: nothing
-// changes for those.)
+// registers once (32 uneven maps 690 -> 659 us). The per-map kernels have both
+// in constant memory; there it gives 0.1 to 0.4 us a pass.
 struct LeanConst {
     float inv_vs, vs, mx, my, mz, ntx, nty, ntz, tau, qs;
     uint32_t omb[3], dmask[3], cy, cz;
@@ -576,6 +568,13 @@ __device__ __forceinline__ void lean_march(const ScanArgs& a, const MapDev& m, i
     }
 }
 
+// One warp: the steps of k-group `grp` (kpt steps) of its 32 rays; the plain
+// atomic and the pool reduction march leanly, the other forms below.
+// SORT (sort reduction, MERGE off): each sample of a lane's ray is written to
+// the ray's pair slot sslot + (its index in the ray's march) instead of being
+// reduced: (voxel word, code) inside the window, kNoVoxel outside. Samples
+// whose slot is at or beyond the capacity (or whose ray has none) take the
+// accumulator reduction instead and set `ovf`.
 template <int MODE, bool MERGE, bool SORT = false, bool POOL = false>
 __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m, unsigned grp, int kpt, const float4 A,
                                              const float4 B, unsigned& hits, unsigned& last_brick,
@@ -653,7 +652,7 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
                     if (MODE == 1) ++hits;
                     *ovf = true;
                 }
-            } else if (MERGE) {
+            } else {   // MERGE
                 if (__ballot_sync(kFull, act) == 0u) continue;   // warp-uniform
                 const unsigned peers = __match_any_sync(kFull, act ? word : kNoVoxel);
                 leader = act && lane == (unsigned)(__ffs(peers) - 1);
@@ -666,13 +665,6 @@ __device__ __forceinline__ void contrib_item(const ScanArgs& a, const MapDev& m,
                     const unsigned key = ((unsigned)abs(q) << 1) | (q < 0 ? 1u : 0u);
                     const unsigned kmin = __reduce_min_sync(peers, key);
                     if (leader) atomicMax(m.acc + word, 65536ull - kmin);
-                }
-            } else {
-                if (MODE == 0) {
-                    if (act) atomicAdd(m.acc + word, (1ull << 40) + (unsigned long long)(long long)q);
-                } else {
-                    const unsigned key = ((unsigned)abs(q) << 1) | (q < 0 ? 1u : 0u);
-                    if (act) atomicMax(m.acc + word, 65536ull - key);
                 }
             }
             if (MODE == 1 && !SORT) hits += act ? 1u : 0u;
@@ -957,27 +949,26 @@ __device__ __forceinline__ void store_pairs(uint2* gp, ulonglong2* ap, const ulo
     }
 }
 
-// ---- apply, register form (batches and the pool reduction): one warp updates
-// grid brick `brick` from the 512 accumulators at `accp` (a brick of the dense
-// accumulator or a pool slot). Lane l holds voxels 2(32 v + l) and +1 as 8-byte
+// ---- apply, register form (batches): one warp updates grid brick `brick` from
+// its accumulators. Lane l holds voxels 2(32 v + l) and +1 as 8-byte
 // grid pairs and 16-byte accumulator pairs, all loaded at once; every touched
 // voxel is decoded in place, and only changed pairs are written back and reset.
 // NV voxel pairs per lane, starting at pair row v0: NV = 8 is the whole
 // brick, NV = 4 (v0 = 0 or 4) one half, NV = 2 a quarter.
 template <int MODE, int NV = 8>
 __device__ __forceinline__ void apply_brick_at(const MapDev& m, int32_t w_max, int32_t flags, unsigned brick,
-                                               unsigned long long* accp, unsigned long long& touched,
-                                               unsigned long long& hits, unsigned v0 = 0) {
+                                               unsigned long long& touched, unsigned long long& hits,
+                                               unsigned v0 = 0) {
     static_assert(NV == 8 || NV == 4 || NV == 2, "whole, half or quarter bricks");
     if constexpr (NV == 8) {   // two halves, one after the other: all sixteen voxels at once would not fit the registers
 #pragma unroll 1
         for (unsigned h = 0; h < 8u; h += 4u)
-            apply_brick_at<MODE, 4>(m, w_max, flags, brick, accp, touched, hits, h);
+            apply_brick_at<MODE, 4>(m, w_max, flags, brick, touched, hits, h);
         return;
     }
     const unsigned lane = threadIdx.x & 31u;
     uint2* gp = reinterpret_cast<uint2*>(m.grid + ((size_t)brick << 9)) + 32 * v0;
-    ulonglong2* ap = reinterpret_cast<ulonglong2*>(accp) + 32 * v0;
+    ulonglong2* ap = reinterpret_cast<ulonglong2*>(m.acc + ((size_t)brick << 9)) + 32 * v0;
     ulonglong2 acc[NV];
     uint2 g[NV];
 #pragma unroll
@@ -993,8 +984,7 @@ template <int MODE, int NV>
 __device__ __forceinline__ void apply_part_reg(const MapDev& m, int32_t w_max, int32_t flags, unsigned t,
                                                unsigned long long& touched, unsigned long long& hits) {
     constexpr unsigned P = 8 / NV;
-    const unsigned brick = m.brick_list[t / P];
-    apply_brick_at<MODE, NV>(m, w_max, flags, brick, m.acc + ((size_t)brick << 9), touched, hits, (t % P) * NV);
+    apply_brick_at<MODE, NV>(m, w_max, flags, m.brick_list[t / P], touched, hits, (t % P) * NV);
 }
 
 // ---- sort reduction (counting sort of the emitted pairs by touched brick,
@@ -1169,8 +1159,8 @@ __device__ __forceinline__ void sort_apply_brick(const MapDev& m, int32_t w_max,
     __syncwarp();
 }
 
-// ---- finish (sort and pool reductions, batches): one warp (lane = counter
-// slot) publishes the scan's counters and clears the per-scan state.
+// ---- finish (sort reduction, batches): one warp (lane = counter slot)
+// publishes the scan's counters and clears the per-scan state.
 __device__ __forceinline__ void finish_warp(const MapDev& m) {
     MapCounters* c = m.ctr;
     const unsigned lane = threadIdx.x & 31u;
@@ -1186,19 +1176,16 @@ __device__ __forceinline__ void finish_warp(const MapDev& m) {
         u += __shfl_xor_sync(kFull, u, o);
     }
     if (lane == 0) {
-        // a pool-reduction scan that found the pool full was dropped
-        const long long st = __ldcg(&c->pool_overflow) != 0u ? kStatusCapacity : 0;
-        if (st != 0) h = u = 0ull;
         c->pub[0] = (long long)v;
         c->pub[1] = (long long)h;
         c->pub[2] = (long long)u;
-        c->pub[3] = st;
+        c->pub[3] = 0;
         c->pub[4] = 0;
         if (m.host_last) {   // also into host memory: reading them needs no copy
             m.host_last[0] = (long long)v;
             m.host_last[1] = (long long)h;
             m.host_last[2] = (long long)u;
-            m.host_last[3] = st;
+            m.host_last[3] = 0;
             m.host_last[4] = 0;
         }
         c->live_count = 0u;
@@ -1206,8 +1193,6 @@ __device__ __forceinline__ void finish_warp(const MapDev& m) {
         c->slot_count = 0ull;
         c->overflow = 0u;
         c->apply_done = 0u;
-        c->pool_count = 0u;
-        c->pool_overflow = 0u;
     }
 }
 
