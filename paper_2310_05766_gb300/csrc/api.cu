@@ -143,7 +143,7 @@ struct tsdf_map {
     bool use_graph = false;
     bool graph_broken = false;      // capture or instantiation failed: plain launches from then on
     bool captured = false;          // a caller has captured a plain scan of this map (see note_capture)
-    cudaStream_t capture_stream = nullptr;
+    cudaStream_t own_stream = nullptr;   // non-blocking: captures, and the filling of new buffers
     struct ScanGraph {
         cudaGraph_t graph = nullptr;
         cudaGraphExec_t exec = nullptr;
@@ -159,6 +159,7 @@ struct tsdf_map {
     long long* host_last = nullptr; // mapped pinned copy of the published counters (host address)
     double* reg_dev = nullptr;      // registration: the CTAs' sums, the 29 sums of the normal equations, a counter
     double reg_serial = 0.0;        // registration: evaluations so far
+    bool reg_clean = false;         // registration: the arrival counter is 0 (the last evaluation completed)
     double* reg_host = nullptr;     // registration: mapped pinned copy of the 29 sums (host address), or null
     RegisterBuffers reg{};
     size_t pair_cap_req = 0;        // sort reduction: requested pair capacity, 0 = from the scan size
@@ -269,7 +270,7 @@ static void chain_graph_reset(tsdf_map::ScanGraph& c) {
 void free_map(tsdf_map* m) {
     if (!m) return;
     for (auto& c : m->chain) chain_graph_reset(c);
-    if (m->capture_stream) cudaStreamDestroy(m->capture_stream);
+    if (m->own_stream) cudaStreamDestroy(m->own_stream);
     for (const Pending& p : m->pending) {
         cudaEventDestroy(p.start);
         cudaEventDestroy(p.stop);
@@ -572,6 +573,7 @@ int tsdf_map_create(const tsdf_params* params, tsdf_map** out) {
         m->host_last = nullptr;
         cudaGetLastError();   // clear a failed mapping request
     }
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&m->own_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->items_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->flags_event, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&m->spill_event, cudaEventDisableTiming);
@@ -592,18 +594,13 @@ int tsdf_map_destroy(tsdf_map* map) {
     return TSDF_OK;
 }
 
-// Fills a new allocation and waits for it, on a stream of its own: the call
+// Fills a new allocation and waits for it, on the map's own stream: the call
 // that needs it may launch on any stream, and a fill on the default stream
 // would be ordered neither before that launch nor apart from what the caller
 // has queued there.
-static cudaError_t fill_new(void* p, int byte, size_t bytes) {
-    cudaStream_t t = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&t, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p, byte, bytes, t);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(t);
-    cudaStreamDestroy(t);
-    return e;
+static cudaError_t fill_new(const tsdf_map* map, void* p, int byte, size_t bytes) {
+    const cudaError_t e = cudaMemsetAsync(p, byte, bytes, map->own_stream);
+    return e == cudaSuccess ? cudaStreamSynchronize(map->own_stream) : e;
 }
 
 // The dense per-scan accumulator (8 B per voxel, all zero between scans) is
@@ -613,7 +610,7 @@ static int ensure_acc(tsdf_map* map) {
     if (map->dev.acc) return TSDF_OK;
     unsigned long long* a = nullptr;
     TSDF_CU(cudaMalloc(&a, map->voxels * sizeof(unsigned long long)));
-    cudaError_t e = fill_new(a, 0, map->voxels * sizeof(unsigned long long));
+    cudaError_t e = fill_new(map, a, 0, map->voxels * sizeof(unsigned long long));
     if (e != cudaSuccess) {
         cudaFree(a);
         return cuda_fail(e);
@@ -642,10 +639,10 @@ static int ensure_pool(tsdf_map* map) {
     map->dev.pool_acc = nullptr;
     map->dev.pool_cap = 0;
     TSDF_CU(cudaMalloc(&map->dev.pool_table, map->bricks * sizeof(uint32_t)));
-    TSDF_CU(fill_new(map->dev.pool_table, 0xFF, map->bricks * sizeof(uint32_t)));
+    TSDF_CU(fill_new(map, map->dev.pool_table, 0xFF, map->bricks * sizeof(uint32_t)));
     TSDF_CU(cudaMalloc(&map->dev.pool_brick, want * sizeof(uint32_t)));
     TSDF_CU(cudaMalloc(&map->dev.pool_acc, want * kBrickVoxels * sizeof(unsigned long long)));
-    TSDF_CU(fill_new(map->dev.pool_acc, 0, want * kBrickVoxels * sizeof(unsigned long long)));
+    TSDF_CU(fill_new(map, map->dev.pool_acc, 0, want * kBrickVoxels * sizeof(unsigned long long)));
     map->dev.pool_cap = (uint32_t)want;
     return TSDF_OK;
 }
@@ -675,7 +672,7 @@ static int ensure_sort(tsdf_map* map, int64_t n) {
         TSDF_CU(cudaMalloc(&map->dev.brick_slot, map->bricks * sizeof(uint32_t)));
         TSDF_CU(cudaMalloc(&map->dev.seg_count, map->bricks * sizeof(uint32_t)));
         TSDF_CU(cudaMalloc(&map->dev.seg_start, map->bricks * sizeof(uint32_t)));
-        TSDF_CU(fill_new(map->dev.seg_count, 0, map->bricks * sizeof(uint32_t)));
+        TSDF_CU(fill_new(map, map->dev.seg_count, 0, map->bricks * sizeof(uint32_t)));
     }
     if (map->ray_slot_cap < map->ray_cap) {
         cudaFree(map->dev.ray_slot);
@@ -751,13 +748,7 @@ static bool same_dev(const MapDev& x, const MapDev& y) {
 // when any step fails (nothing is left half built).
 static bool chain_graph_build(tsdf_map* map, tsdf_map::ScanGraph& c, const ScanArgs& a) {
     chain_graph_reset(c);
-    if (!map->capture_stream &&
-        cudaStreamCreateWithFlags(&map->capture_stream, cudaStreamNonBlocking) != cudaSuccess) {
-        map->capture_stream = nullptr;
-        cudaGetLastError();
-        return false;
-    }
-    cudaStream_t cs = map->capture_stream;
+    cudaStream_t cs = map->own_stream;
     if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -1613,11 +1604,6 @@ static int ensure_register(tsdf_map* map) {
     static_assert(kRegisterBytes == (kSums + 32 + 1) * sizeof(double), "sums, system, counter");
     double* d = nullptr;
     TSDF_CU(cudaMalloc(&d, kRegisterBytes));
-    cudaError_t e = fill_new(d, 0, kRegisterBytes);
-    if (e != cudaSuccess) {
-        cudaFree(d);
-        return cuda_fail(e);
-    }
     map->reg.part = d;
     map->reg.out = d + kSums;
     map->reg.done = reinterpret_cast<unsigned*>(d + kSums + 32);
@@ -1651,12 +1637,17 @@ static int register_evaluate(tsdf_map* map, const float* points_dev, int64_t n, 
                              int32_t min_weight, double* out_host, cudaStream_t s) {
     int rc = ensure_register(map);
     if (rc != TSDF_OK) return rc;
+    // the arrival counter starts at 0 and every complete evaluation leaves it so
+    // (on this stream: the kernel below is ordered behind it)
+    if (!map->reg_clean) TSDF_CU(cudaMemsetAsync(map->reg.done, 0, sizeof(unsigned), s));
+    map->reg_clean = false;
     const long long o[3] = {map->origin[0], map->origin[1], map->origin[2]};
     TSDF_CU(launch_register(points_dev, (int)n, pose, map->dev.grid, map->geom, o, map->p.voxel_size, map->inv_vs,
                             map->p.tau, min_weight, map->num_sms, map->reg, ++map->reg_serial, s));
     if (!map->reg_host) {
         TSDF_CU(cudaMemcpyAsync(out_host, map->reg.out, 29 * sizeof(double), cudaMemcpyDeviceToHost, s));
         TSDF_CU(cudaStreamSynchronize(s));
+        map->reg_clean = true;
         return TSDF_OK;
     }
     // The kernel's last CTA writes the serial behind the sums: watching it for
@@ -1671,6 +1662,7 @@ static int register_evaluate(tsdf_map* map, const float* points_dev, int64_t n, 
     std::atomic_thread_fence(std::memory_order_acquire);
     if (*mark != map->reg_serial) TSDF_CU(cudaStreamSynchronize(s));
     if (*mark != map->reg_serial) return cuda_fail(cudaErrorUnknown);   // the sums are not this evaluation's
+    map->reg_clean = true;
     std::memcpy(out_host, map->reg_host, 29 * sizeof(double));
     return TSDF_OK;
 }
