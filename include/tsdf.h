@@ -269,7 +269,8 @@ int tsdf_stats(tsdf_map* map, tsdf_scan_stats* out, void* stream);
                                       host memory at the next shift; 0 (default): only when the device tier is
                                       full */
 #define TSDF_OPT_LAUNCH_GRAPH 10  /* 1: the atomic reduction's two to four kernels are captured once into a CUDA
-                                    graph (again after buffers or options change) and each scan sets the
+                                    graph (one for scans of up to 32768 points and one for larger ones; again
+                                    after buffers or options change) and each scan sets the
                                     graph's arguments and launches it once: less host time per scan, for
                                     callers whose thread is the bottleneck; 0 (default): one launch per
                                     kernel, which lets consecutive scans overlap on the device. Scans while
@@ -449,7 +450,9 @@ typedef struct tsdf_batch tsdf_batch;   /* opaque; owns pinned and device descri
 #define TSDF_BATCH_OPT_SPIN_LIMIT 4  /* polls before a grid-barrier wait gives up (default 2^24, about a second) */
 #define TSDF_BATCH_OPT_TEST_MISSING_ARRIVALS 5  /* test hook: the barrier waits for this many CTAs that do not exist (default 0) */
 #define TSDF_BATCH_OPT_GRID_FRACTION 6  /* percent (1..100, default 100) of the device's co-resident CTAs the launch uses,
-                                           so that launches on several streams can be resident together */
+                                           so that launches on several streams can be resident together (a plain
+                                           tsdf_integrate on another stream waits for launches of the 128-thread
+                                           configurations, which leave its last kernel no room) */
 #define TSDF_BATCH_OPT_TUNE_SORT  7  /* 1 (default): the autotuner also times the sort configurations, whose first use
                                         allocates each map's sort buffers; 0: only the atomic ones (no allocation) */
 #define TSDF_BATCH_OPT_CTA_BRICK_CACHE 8  /* 1 (default): the warps of a CTA share one cache of the bricks they

@@ -137,9 +137,9 @@ struct tsdf_map {
     // The plain path's launches as a CUDA graph (TSDF_OPT_LAUNCH_GRAPH):
     // captured on first use, then per scan the ray and contribution nodes get
     // the scan's arguments and the graph is launched once. Off by default: it
-    // cuts the host's time per scan from about 9 to 3.5 us, but back-to-back
-    // scans took 28.8 instead of 26.1 us on the device (the programmatic
-    // overlap of one scan's last kernel with the next scan's first is lost).
+    // cuts the host's time per scan (through the Python binding from 15 to 10.5
+    // us), but back-to-back scans take 28.7 instead of 23.3 us on the device (the
+    // overlap of one scan's apply with the next scan's ray set-up is lost).
     bool use_graph = false;
     bool graph_broken = false;      // capture or instantiation failed: plain launches from then on
     bool captured = false;          // a caller has captured a plain scan of this map (see note_capture)

@@ -77,13 +77,18 @@
 #ifndef TSDF_CONTRIB_MIN_CTAS
 #define TSDF_CONTRIB_MIN_CTAS 4
 #endif
-// Largest scan of the one-kernel path (points). Above it a scan's tiles differ
-// too much in cost for the chip to be filled evenly by whole tiles, and the
-// global ray list, whose 32-ray blocks all march, is the better one. Passes of
-// both paths, one kernel / ray list, in us: room 16x360 17.9 / 26.2 and 64x512
-// 17.2 / 18.1; outdoor 16x512 21.1 / 33.1, 32x512 18.6 / 24.6, 32x1024 34.3 /
-// 38.0, 64x1024 31.3 / 29.4, 128x1024 30.0 / 26.9; corridor 32x512 38.5 / 49.5,
-// 64x1024 41.9 / 44.9, 128x2048 52.1 / 51.4.
+// Largest scan of the one-kernel path (points). Drawn when the other path was
+// four kernels (one kernel / ray list, us a pass: room 16x360 17.9 / 26.2 and
+// 64x512 17.2 / 18.1; outdoor 16x512 21.1 / 33.1, 32x512 18.6 / 24.6, 64x1024
+// 31.3 / 29.4; corridor 32x512 38.5 / 49.5, 64x1024 41.9 / 44.9). With the ray
+// set-up beside the previous scan's apply the list has become the faster one for
+// most scans that follow one another: room 16x360 14.2 / 14.4 and 64x512 14.0 /
+// 14.4; outdoor 16x512 29.2 / 26.0, 32x512 25.8 / 23.1, 32x1024 31.2 / 26.7,
+// 64x1024 29.6 / 24.7, 128x1024 27.6 / 23.2; corridor 32x512 32.3 / 28.7, 32x1024
+// 37.1 / 33.9, 64x1024 35.6 / 34.3, 128x2048 46.2 / 41.6. Scans alone (wall time
+// of the call and its end): room 16x360 31.1 / 31.1, outdoor 32x512 44.5 / 43.7,
+// corridor 32x512 50.8 / 49.4; the static entry 21.3-23.8 / 22.6. The one-kernel
+// path needs no ray buffers.
 #ifndef TSDF_SCAN_FUSED_MAX
 #define TSDF_SCAN_FUSED_MAX 32768
 #endif
@@ -448,7 +453,10 @@ constexpr int kApplyWarps = 4;   // CTA size of the sort reduction's apply kerne
 // Before (compaction kernel, four CTAs of 128 threads per SM and more, no
 // staging, counters through the last CTA): outdoor 26.8, corridor 51.4, box room
 // 17.9 us a pass; so staged: 23.1, 46.2, 14.4; with the exact quotient of
-// apply_voxel_fast in place of an integer division 22.2, 45.5, 14.3.
+// apply_voxel_fast in place of an integer division 22.2, 45.5, 14.3. Its 36.9 k
+// registers find no room beside three CTAs of 128 threads of a batched launch;
+// with 64 registers a thread it would, but then two CTAs fit an SM and land on
+// it (outdoor 27, corridor 52), and with 384 threads at 25.3 and 52.
 constexpr int kApplyThreads = 512;
 constexpr int kApplyWarpsPlain = kApplyThreads / 32;
 constexpr int kApplyStages = 4;
@@ -457,6 +465,11 @@ constexpr unsigned kApplyParts = 8u / kApplyPairs;
 constexpr int kStageBytes = 128 * (8 + 4);        // accumulators and grid words of a quarter brick
 constexpr int kApplySmem = kApplyWarpsPlain * kApplyStages * kStageBytes;
 constexpr int kApplyList = 1024;                  // bricks of one CTA listed at a time
+// Windows whose flags every CTA reads itself; larger ones go through the
+// compaction kernel. Flags / list, us a pass: 2^16 bricks 23.5 / 24.5 (outdoor
+// 128x1024) and 29.2 / 30.0 (16x512), 2^17 bricks 26.1 / 24.4 and 32.3 / 30.4;
+// with flags up to 2^17 a thread holds 16 vectors of them and windows of 2^15
+// take 18.8 instead of 17.3.
 constexpr uint32_t kFlagBricks = 1u << 16;
 constexpr int kFlagVecs = (int)(kFlagBricks / 16) / kApplyThreads;   // 16-flag vectors per thread, at most
 static_assert(kFlagVecs * kApplyThreads * 16 == (int)kFlagBricks && kFlagVecs % 2 == 0, "flags per thread");

@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(kRegWarps * 32) register_kernel(const RegArgs 
 
 // CTAs of the kernel: one of six warps per SM. The binary64 unit is full with
 // that, and a thread of a 128 x 1024 scan adds up four or five points before
-// the warp's sums (six evaluations and one more: 239 us; eight warps 250, two
-// CTAs per SM 262-273 us; 720 us before).
+// the warp's sums (six evaluations and one more: 239 us, 234-255 since the two
+// calls synchronise; eight warps 250, two CTAs per SM 262-273 us; 720 us before).
 cudaError_t launch_register(const float* pts_dev, int n, const float pose[12], const uint32_t* grid,
                             const WindowGeom& geo, const long long origin[3], float vs, float inv_vs, float tau,
                             int min_w, int sms, const RegisterBuffers& buf, double serial, cudaStream_t s) {
